@@ -412,11 +412,15 @@ __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm
     return best;
 }
 
+// A triangle as the traversal reaches it: 2 * node + child for a leaf of the
+// binary hierarchy, -2 - k for large triangle k, RT_NO_REF for none.
+#define RT_NO_REF (-1)
+
 // Any occluder on the open segment (tmin, tmax) along o + t d (d unit),
-// skipping original ids ex0 / ex1.
-template <bool C, bool V8>
+// skipping original ids ex0 / ex1. REF: the occluder found goes to ref.
+template <bool C, bool V8, bool REF = false>
 __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, int n_sm, f3 o, f3 d,
-                                          float tmax, int ex0, int ex1, TravCount& cnt) {
+                                          float tmax, int ex0, int ex1, TravCount& cnt, int* ref = nullptr) {
     if (C) cnt.queries++;
     if (s.n_tris == 0) return false;
     f3 inv = safe_inv(d);
@@ -432,7 +436,10 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
         int id = __float_as_int(r0.w);
         if (id != ex0 && id != ex1) {
             float t = tri_hit(r0, r1, r2, o, d);
-            if (t > tmin && t < tmax) return true;
+            if (t > tmin && t < tmax) {
+                if (REF) *ref = -2 - k;
+                return true;
+            }
         }
     }
     const float4* onodes = octant_nodes(s, inv);
@@ -452,7 +459,10 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
             int id = __float_as_int(r0.w);
             if (id != ex0 && id != ex1) {
                 float t = tri_hit(r0, r1, r2, o, d);
-                if (t > tmin && t < tmax) return true;
+                if (t > tmin && t < tmax) {
+                    if (REF) *ref = 2 * node + 0;
+                    return true;
+                }
             }
             h0 = false;
         }
@@ -463,7 +473,10 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
             int id = __float_as_int(r0.w);
             if (id != ex0 && id != ex1) {
                 float t = tri_hit(r0, r1, r2, o, d);
-                if (t > tmin && t < tmax) return true;
+                if (t > tmin && t < tmax) {
+                    if (REF) *ref = 2 * node + 1;
+                    return true;
+                }
             }
             h1 = false;
         }
@@ -480,6 +493,34 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
         }
     }
     return false;
+}
+
+// Whether the triangle `ref` (from an earlier any_hit_b) occludes this segment:
+// one box test and one triangle test instead of a traversal. True exactly
+// where the traversal would report this triangle as a hit: it reaches a leaf
+// whose own box is hit, since every ancestor's planes enclose the leaf's and
+// a plane's distance (one FMA, rounded once) is monotone in the plane.
+__device__ __forceinline__ bool ref_hit(const DevScene& s, int ref, f3 o, f3 d, float tmax, int ex0, int ex1) {
+    if (ref == RT_NO_REF) return false;
+    const float4* tp;
+    if (ref < 0) {
+        tp = s.big + 3 * (size_t)(-2 - ref);
+    } else {
+        const f3 inv = safe_inv(d);
+        const f3 oi = {o.x * inv.x, o.y * inv.y, o.z * inv.z};
+        float4 a, b, c, e;
+        load_node<true>(octant_nodes(s, inv) + 4 * (size_t)(ref >> 1), a, b, c, e);
+        float tn0, tf0, tn1, tf1;
+        box_pair(a, b, c, pair_ray(inv, oi), s.tmin, tmax, tn0, tf0, tn1, tf1);
+        const bool second = ref & 1;
+        if (!((second ? tn1 : tn0) <= (second ? tf1 : tf0))) return false;
+        tp = s.tris + 3 * (size_t)(~__float_as_int(second ? e.y : e.x));
+    }
+    const float4 r0 = ldg4(tp), r1 = ldg4(tp + 1), r2 = ldg4(tp + 2);
+    const int id = __float_as_int(r0.w);
+    if (id == ex0 || id == ex1) return false;
+    const float t = tri_hit(r0, r1, r2, o, d);
+    return t > s.tmin && t < tmax;
 }
 
 // Closest hit on the 8-wide layout; same contract as closest_hit_b.

@@ -48,9 +48,12 @@ struct CellGrid {
     int nx, ny;
 };
 
-__device__ __forceinline__ f3 cell_centre(const CellGrid& g, int64_t r) {
-    const int64_t iy = r / g.nx, ix = r - iy * g.nx;
+__device__ __forceinline__ f3 cell_centre(const CellGrid& g, int ix, int iy) {
     return mk(g.x0 + ((float)ix + 0.5f) * g.cell, g.y0 + ((float)iy + 0.5f) * g.cell, g.h);
+}
+__device__ __forceinline__ f3 cell_centre(const CellGrid& g, int64_t r) {
+    const int iy = (int)r / g.nx;   // a map has fewer than 2^31 cells
+    return cell_centre(g, (int)r - iy * g.nx, iy);
 }
 
 struct DiffFind {
@@ -61,7 +64,7 @@ struct DiffFind {
     const float* rx_pos;
     const int32_t* rx_off;   // [n_tx+1] or null
     int n_tx, n_rx;
-    int64_t total;           // pairs * wedges
+    int tiles, runs;         // receiver tiles of 32 (of the largest receiver set), runs of DF_RUN tiles
     CellGrid grid;           // receivers at cell centres when grid.nx > 0
     unsigned long long* count;
     unsigned long long cap;
@@ -85,50 +88,188 @@ __device__ __forceinline__ void pair_devices(const int32_t* rx_off, int n_tx, in
     }
 }
 
-// One thread per (pair, wedge): Keller point, exterior test, two segment
-// occlusion tests; valid paths are appended (order fixed afterwards by a sort).
+// Any occluder (any_hit), with the one found in `found` on the binary layout
+// (RT_NO_REF on the wide one, whose leaves have no such reference).
 template <int LY>
-__global__ void __launch_bounds__(256) k_diff_find(DiffFind p) {
+__device__ __forceinline__ bool any_hit_ref(const DevScene& s, f3 o, f3 d, float tmax, int ex0, int ex1,
+                                            TravCount& cnt, int& found) {
+    if (LY == 8) return any_hit<false, 8>(s, nullptr, 0, o, d, tmax, ex0, ex1, cnt);
+    return any_hit_b<false, true, true>(s, nullptr, 0, o, d, tmax, ex0, ex1, cnt, &found);
+}
+
+// D -> rx of the last (up to 32) of a warp's n2 queued candidates; the open
+// ones are paths. Called by all 32 lanes.
+template <int LY>
+__device__ __forceinline__ void diff_tail(const DiffFind& p, const int* qr, const float* qt, int& n2, int t, int wi,
+                                          f3 A, f3 e, int f0, int f1, int& ref2, TravCount& cnt) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int take = min(n2, 32);
+    n2 -= take;
+    bool open = false;
+    int found = RT_NO_REF, r = 0;
+    f3 D = mk(0.0f, 0.0f, 0.0f);
+    if (lane < take) {
+        r = qr[n2 + lane];
+        D = A + e * qt[n2 + lane];
+        const f3 rx = p.grid.nx > 0 ? cell_centre(p.grid, r) : mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
+        const f3 d = rx - D;
+        const float L = sqrtf(dot(d, d));
+        open = !any_hit_ref<LY>(p.s, D, d * (1.0f / L), L - p.s.tmin, f0, f1, cnt, found);
+    }
+    const unsigned fm = __ballot_sync(full, found != RT_NO_REF);
+    if (fm) ref2 = __shfl_sync(full, found, 31 - __clz(fm));
+    const unsigned m = __ballot_sync(full, open);
+    if (m) {
+        const int leader = __ffs(m) - 1;
+        unsigned long long b0 = 0;
+        if (lane == leader) b0 = atomicAdd(p.count, (unsigned long long)__popc(m));
+        b0 = __shfl_sync(full, b0, leader);
+        const unsigned long long k = b0 + __popc(m & lanemask_lt());
+        if (open && k < p.cap) {
+            const uint64_t pair = p.rx_off ? (uint64_t)r : (uint64_t)t * (uint64_t)p.n_rx + (uint64_t)r;
+            p.keys[k] = (pair << 32) | (uint64_t)wi;
+            p.pts[k] = make_float4(D.x, D.y, D.z, 0.0f);
+        }
+    }
+    __syncwarp();
+}
+
+// Receiver tiles of a work unit, and cells of a grid tile (8 x 4: neighbouring
+// cells see a wedge past the same occluders).
+constexpr int DF_RUN = 64;
+constexpr int DF_TX = 8, DF_TY = 4;
+constexpr int DF_Q = 64;   // entries of a warp's queues
+
+// Every (transmitter, wedge, receiver): Keller point, exterior test, two
+// segment occlusion tests; valid paths are appended (order fixed afterwards
+// by a sort). A warp takes one wedge and one transmitter against a run of
+// receiver tiles, a lane per receiver, so the wedge's record, its exterior
+// normal and the transmitter's side of Keller's law are computed once per run
+// and neighbouring lanes test nearby segments. The occluder that last blocked
+// tx -> D (and D -> rx) for this run is tried first (ref_hit: one box and one
+// triangle instead of a traversal); the candidates it does not block are
+// queued, so that the traversals run with all 32 lanes.
+//
+// Bound by the candidates' own arithmetic and by the segments no kept
+// occluder answers. City map of 500 x 500 cells x 4800 wedges (1.2e9
+// candidates): 73.3 ms with one thread per (receiver, wedge) in wedge order
+// (7.6 of 32 lanes active, the wedge reloaded and its sincos and transmitter
+// side recomputed per candidate), 12.6 ms now.
+template <int LY>
+__global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
+    __shared__ int q1r[4][DF_Q], q2r[4][DF_Q];
+    __shared__ float q1t[4][DF_Q], q2t[4][DF_Q];
+    const unsigned full = 0xffffffffu, lt = lanemask_lt();
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int64_t units = (int64_t)p.n_tx * p.runs * p.n_w;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const bool map = p.grid.nx > 0;
+    const int tiles_y = (p.grid.ny + DF_TY - 1) / DF_TY;
     TravCount cnt;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < p.total;
-         u += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t pair = u / p.n_w;
-        const int wi = (int)(u - pair * p.n_w);
-        int t;
-        int64_t r;
-        pair_devices(p.rx_off, p.n_tx, p.n_rx, pair, t, r);
+    for (int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + wp; u < units; u += step) {
+        const int64_t tr_ = u / p.n_w;
+        const int wi = (int)(u - tr_ * p.n_w);
+        const int t = (int)(tr_ / p.runs), run = (int)(tr_ - (int64_t)t * p.runs);
+        const int r0 = p.rx_off ? p.rx_off[t] : 0;
+        const int R = p.rx_off ? p.rx_off[t + 1] - r0 : p.n_rx;
         const WedgeDev w = p.w[wi];
         const f3 A = xyz(w.a), e = xyz(w.e);
         const f3 tx = mk(p.tx_pos[3 * t], p.tx_pos[3 * t + 1], p.tx_pos[3 * t + 2]);
-        const f3 rx = p.grid.nx > 0 ? cell_centre(p.grid, r)
-                                    : mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
-        const float ts = dot(tx - A, e), tr = dot(rx - A, e);
-        const f3 ps = tx - A - e * ts, pr = rx - A - e * tr;
-        const float rs = sqrtf(dot(ps, ps)), rr = sqrtf(dot(pr, pr));
-        if (!(rs + rr > 0.0f)) continue;
-        const float tpar = ts + (tr - ts) * (rs / (rs + rr));
-        if (!(tpar > 0.0f && tpar < w.a.w)) continue;
-        const f3 D = A + e * tpar;
+        const float ts = dot(tx - A, e);
+        const f3 ps = tx - A - e * ts;
+        const float rs = sqrtf(dot(ps, ps));
         // outside the solid: on the exterior side of face 0 (v . n0 > 0) or of
         // face 1, whose exterior normal is sin(n pi) t0 - cos(n pi) n0
         float sn, cn;
         sincospif(w.e.w, &sn, &cn);
-        const f3 vt = tx - D, vr = rx - D;
-        const float yt = dot(vt, xyz(w.n0)), yr = dot(vr, xyz(w.n0));
-        const bool out_t = yt > 0.0f || sn * dot(vt, xyz(w.t0)) - cn * yt > 0.0f;
-        const bool out_r = yr > 0.0f || sn * dot(vr, xyz(w.t0)) - cn * yr > 0.0f;
-        if (!(out_t && out_r)) continue;
         const int f0 = __float_as_int(w.t0.w), f1 = __float_as_int(w.n0.w);
-        f3 d = D - tx;
-        float L = sqrtf(dot(d, d));
-        if (any_hit<false, LY>(p.s, nullptr, 0, tx, d * (1.0f / L), L - p.s.tmin, f0, f1, cnt)) continue;
-        d = rx - D;
-        L = sqrtf(dot(d, d));
-        if (any_hit<false, LY>(p.s, nullptr, 0, D, d * (1.0f / L), L - p.s.tmin, f0, f1, cnt)) continue;
-        const unsigned long long k = atomicAdd(p.count, 1ull);
-        if (k < p.cap) {
-            p.keys[k] = ((uint64_t)pair << 32) | (uint64_t)wi;
-            p.pts[k] = make_float4(D.x, D.y, D.z, 0.0f);
+        int ref1 = RT_NO_REF, ref2 = RT_NO_REF;   // last occluders of tx -> D and D -> rx
+        int n1 = 0, n2 = 0;                       // queued candidates (warp-uniform)
+        const int tile_end = min(p.tiles, (run + 1) * DF_RUN);
+        for (int tile = run * DF_RUN; tile <= tile_end; tile++) {
+            const bool last = tile == tile_end;   // one more turn empties the queues
+            bool open1 = false;
+            int r = 0;
+            float tpar = 0.0f;
+            if (!last) {
+                bool in;
+                f3 rx;
+                if (map) {
+                    const int cx = tile / tiles_y, cy = tile - cx * tiles_y;
+                    const int ix = cx * DF_TX + (lane & (DF_TX - 1)), iy = cy * DF_TY + lane / DF_TX;
+                    in = ix < p.grid.nx && iy < p.grid.ny;
+                    r = iy * p.grid.nx + ix;
+                    rx = cell_centre(p.grid, ix, iy);
+                } else {
+                    r = 32 * tile + lane;
+                    in = r < R;
+                    r += r0;
+                    if (in) rx = mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
+                }
+                if (in) {
+                    const float tr = dot(rx - A, e);
+                    const f3 pr = rx - A - e * tr;
+                    const float rr = sqrtf(dot(pr, pr));
+                    tpar = ts + (tr - ts) * (rs / (rs + rr));
+                    if (rs + rr > 0.0f && tpar > 0.0f && tpar < w.a.w) {
+                        const f3 D = A + e * tpar;
+                        const f3 vt = tx - D, vr = rx - D;
+                        const float yt = dot(vt, xyz(w.n0)), yr = dot(vr, xyz(w.n0));
+                        const bool out_t = yt > 0.0f || sn * dot(vt, xyz(w.t0)) - cn * yt > 0.0f;
+                        const bool out_r = yr > 0.0f || sn * dot(vr, xyz(w.t0)) - cn * yr > 0.0f;
+                        if (out_t && out_r) {
+                            const f3 d = D - tx;
+                            const float L = sqrtf(dot(d, d));
+                            open1 = !ref_hit(p.s, ref1, tx, d * (1.0f / L), L - p.s.tmin, f0, f1);
+                        }
+                    }
+                }
+            }
+            const unsigned m1 = __ballot_sync(full, open1);
+            if (open1) {
+                const int k = n1 + __popc(m1 & lt);
+                q1r[wp][k] = r;
+                q1t[wp][k] = tpar;
+            }
+            n1 += __popc(m1);
+            __syncwarp();
+            while (n1 >= 32 || (last && n1 > 0)) {
+                // tx -> D of up to 32 queued candidates
+                const int take = min(n1, 32);
+                n1 -= take;
+                bool open2 = false;
+                int found = RT_NO_REF;
+                if (lane < take) {
+                    r = q1r[wp][n1 + lane];
+                    tpar = q1t[wp][n1 + lane];
+                    const f3 D = A + e * tpar;
+                    f3 d = D - tx;
+                    float L = sqrtf(dot(d, d));
+                    open2 = !any_hit_ref<LY>(p.s, tx, d * (1.0f / L), L - p.s.tmin, f0, f1, cnt, found);
+                    if (open2) {
+                        const f3 rx = map ? cell_centre(p.grid, r) : mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
+                        d = rx - D;
+                        L = sqrtf(dot(d, d));
+                        open2 = !ref_hit(p.s, ref2, D, d * (1.0f / L), L - p.s.tmin, f0, f1);
+                    }
+                }
+                unsigned fm = __ballot_sync(full, found != RT_NO_REF);
+                if (fm) ref1 = __shfl_sync(full, found, 31 - __clz(fm));
+                const unsigned m2 = __ballot_sync(full, open2);
+                if (open2) {
+                    const int k = n2 + __popc(m2 & lt);
+                    q2r[wp][k] = r;
+                    q2t[wp][k] = tpar;
+                }
+                n2 += __popc(m2);
+                __syncwarp();
+                if (n2 >= 32 || (last && n1 == 0 && n2 > 0)) {
+                    diff_tail<LY>(p, q2r[wp], q2t[wp], n2, t, wi, A, e, f0, f1, ref2, cnt);
+                }
+            }
+            if (last)
+                while (n2 > 0) diff_tail<LY>(p, q2r[wp], q2t[wp], n2, t, wi, A, e, f0, f1, ref2, cnt);
         }
     }
 }
@@ -337,6 +478,17 @@ __global__ void __launch_bounds__(64) k_diff_field(DiffField c, float2* __restri
 
 }  // namespace
 
+static void launch_diff_find(rt_ctx* ctx, DiffFind& p) {
+    p.runs = (p.tiles + DF_RUN - 1) / DF_RUN;
+    const int64_t units = (int64_t)p.n_tx * p.runs * p.n_w;
+    const auto kern = wide_layout(ctx) ? k_diff_find<8> : k_diff_find<2>;
+    const int64_t fit = (int64_t)std::max(1, blocks_per_sm((const void*)kern, 128, 0)) * ctx->num_sms;
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((units + 3) / 4, fit));
+    prof_begin(ctx, "k_diff_find");
+    kern<<<(unsigned)blocks, 128, 0, ctx->stream>>>(p);
+    prof_end(ctx);
+}
+
 // Wedges of the current scene, built on the host from the input vertices the
 // first time diffraction is asked for after a scene load.
 static int build_wedges(rt_ctx* ctx) {
@@ -436,8 +588,13 @@ int diffraction_impl(rt_ctx* ctx, int64_t* n_out) {
     p.rx_off = ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr;
     p.n_tx = ctx->n_tx;
     p.n_rx = ctx->n_rx;
-    p.total = total;
     p.grid = CellGrid{0.0f, 0.0f, 0.0f, 0.0f, 0, 0};
+    int r_max = ctx->n_rx;
+    if (ctx->rx_sets) {
+        r_max = 0;
+        for (int t = 0; t < ctx->n_tx; t++) r_max = std::max(r_max, ctx->rx_off[t + 1] - ctx->rx_off[t]);
+    }
+    p.tiles = (r_max + 31) / 32;
     unsigned long long cap = std::max<unsigned long long>(1ull << 14, (unsigned long long)ctx->dpath_cap);
     unsigned long long found = 0;
     for (int attempt = 0; attempt < 2; attempt++) {
@@ -448,10 +605,7 @@ int diffraction_impl(rt_ctx* ctx, int64_t* n_out) {
         p.cap = cap;
         p.keys = bp<uint64_t>(ctx->dpath_raw_key);
         p.pts = bp<float4>(ctx->dpath_raw_pt);
-        const int64_t grid = std::min<int64_t>((total + 255) / 256, 8 * (int64_t)ctx->num_sms);
-        prof_begin(ctx, "k_diff_find");
-        (wide_layout(ctx) ? k_diff_find<8> : k_diff_find<2>)<<<(unsigned)grid, 256, 0, st>>>(p);
-        prof_end(ctx);
+        launch_diff_find(ctx, p);
         RT_TRY(cudaGetLastError());
         RT_TRY(cudaMemcpyAsync(ctx->host_rb, ctx->counters.p, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
         RT_TRY(cudaStreamSynchronize(st));
@@ -588,8 +742,8 @@ int diffraction_map_impl(rt_ctx* ctx, const rt_grid* g, int tx_port, float* gain
     p.rx_off = nullptr;
     p.n_tx = ctx->n_tx;
     p.n_rx = (int)cells;
-    p.total = total;
     p.grid = grid;
+    p.tiles = ((g->nx + DF_TX - 1) / DF_TX) * ((g->ny + DF_TY - 1) / DF_TY);
     unsigned long long cap = std::max<unsigned long long>(1ull << 16, (unsigned long long)ctx->dmap_cap);
     unsigned long long found = 0;
     for (int attempt = 0; attempt < 2; attempt++) {
@@ -600,10 +754,7 @@ int diffraction_map_impl(rt_ctx* ctx, const rt_grid* g, int tx_port, float* gain
         p.cap = cap;
         p.keys = bp<uint64_t>(ctx->dmap_key);
         p.pts = bp<float4>(ctx->dmap_pt);
-        const int64_t blocks = std::min<int64_t>((total + 255) / 256, 8 * (int64_t)ctx->num_sms);
-        prof_begin(ctx, "k_diff_find");
-        (wide_layout(ctx) ? k_diff_find<8> : k_diff_find<2>)<<<(unsigned)blocks, 256, 0, st>>>(p);
-        prof_end(ctx);
+        launch_diff_find(ctx, p);
         RT_TRY(cudaGetLastError());
         RT_TRY(cudaMemcpyAsync(ctx->host_rb, ctx->counters.p, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
         RT_TRY(cudaStreamSynchronize(st));
