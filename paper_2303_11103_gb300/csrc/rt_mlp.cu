@@ -306,7 +306,9 @@ __global__ void k_head_bwd(const __nv_bfloat16* __restrict__ H, const float* __r
 // of the staged dZ for the bias, in 8 interleaved sums (all 128 columns in one
 // CTA of a layer held the others up: 126 us).
 // Bound by what an SM takes in (20 KB per 64 rows: 5.2 MB per CTA at B =
-// 16384); eight stages cover the L2 latency: WG_MEASURED
+// 16384); eight stages cover the L2 latency. B = 16384, W = 256, L = 8: 97 us,
+// where transposed copies, a GEMM per layer and a column sum per layer took
+// 1.3 ms.
 constexpr int WG_ROWS = 64, WG_ST = 8, WG_N = 32;
 constexpr uint32_t WG_CHUNK = WG_ROWS * 128;            // 64 rows x 64 columns of dZ
 constexpr uint32_t WG_STAGE = 2 * WG_CHUNK + WG_ROWS * WG_N * 2;
@@ -839,7 +841,8 @@ __global__ void __launch_bounds__(FM_THREADS, 1) k_mlp_fused(const __grid_consta
 // and order, same sums in the head and the loss). Every wait is bounded; after
 // a timeout the roles run on without waiting, on the same control flow.
 // One tile per CTA: 128 CTAs at B = 16384, and the per-pass latency (first
-// chunk's epilogue + four chunks of MMA) bounds it: TC_MEASURED
+// chunk's epilogue + four chunks of MMA) bounds it: 67 us for B = 16384,
+// W = 256, L = 8, where a kernel per layer and step took 1.0 ms.
 constexpr int TC_THREADS = 352;
 struct TrainArgs {
     const float* x;        // [B x 6]
@@ -1555,17 +1558,17 @@ int rt_mlp_train_step(rt_mlp* m, const float* x, const float* target, int32_t B,
         rc = launch_train_chain(m, x, target, B, loss, NS);
         if (rc) return rc;
     } else {
-    rc = mlp_forward(m, x, B);
-    if (rc) return rc;
-    k_loss<<<(B + 255) / 256, 256, 0, st>>>(bp<float>(m->y), target, x, B, m->db_scale, m->db_offset, m->lam,
-                                           bp<float>(m->dy), loss);
-    auto dz = [&](int l) { return bp<__nv_bfloat16>(m->dZ) + (size_t)l * m->cap * W; };
-    k_head_bwd<<<B / HB_ROWS, W / 2, 0, st>>>(m->hid(L), bp<float>(m->dy), W, m->wp(L), dz(L - 1),
-                                              bp<float>(m->hpart));
-    MT(cudaGetLastError());
-    // dH_l = dZ_l W_l, then through the ReLU of layer l's input
-    for (int l = L - 1; l > 0; l--)
-        MT(gemm_bf16(st, dz(l), m->wtb(l), B, W, W, nullptr, 0, 1, dz(l - 1), W, err, m->hid(l)));
+        rc = mlp_forward(m, x, B);
+        if (rc) return rc;
+        k_loss<<<(B + 255) / 256, 256, 0, st>>>(bp<float>(m->y), target, x, B, m->db_scale, m->db_offset, m->lam,
+                                               bp<float>(m->dy), loss);
+        auto dz = [&](int l) { return bp<__nv_bfloat16>(m->dZ) + (size_t)l * m->cap * W; };
+        k_head_bwd<<<B / HB_ROWS, W / 2, 0, st>>>(m->hid(L), bp<float>(m->dy), W, m->wp(L), dz(L - 1),
+                                                  bp<float>(m->hpart));
+        MT(cudaGetLastError());
+        // dH_l = dZ_l W_l, then through the ReLU of layer l's input
+        for (int l = L - 1; l > 0; l--)
+            MT(gemm_bf16(st, dz(l), m->wtb(l), B, W, W, nullptr, 0, 1, dz(l - 1), W, err, m->hid(l)));
     }
     // dW_l = dZ_l^T H_l and the bias gradients of all hidden layers
     WgradArgs wa;

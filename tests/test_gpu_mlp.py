@@ -148,3 +148,37 @@ def test_surrogate_save_load_roundtrip():
         rt.Surrogate.load(bytes(bad))
     S.close()
     S2.close()
+
+
+@pytest.mark.parametrize("F,W,L,B,first", [(32, 64, 1, 128, 0),       # one layer: no backward pass
+                                           (32, 192, 2, 384, 1000),   # 1000 rows reserved before: layers 1000 rows apart
+                                           (64, 128, 3, 128 * 153, 0),   # more tiles than SMs
+                                           (12, 64, 2, 256, 0),       # features in no whole 64-column chunk: layer by layer
+                                           (64, 256, 16, 128, 0)])    # the deepest and widest
+def test_train_step_shapes(F, W, L, B, first):
+    """Loss and gradients of one step against the CPU reference at the edges of
+    the training kernels' ranges. Tolerance: a BF16 rounding (2^-9 relative)
+    that falls the other way in each layer, forward and backward."""
+    tol = 2 * L * 2.0 ** -9
+    lo = np.array([-250, -250, 0, -250, -250, 0], np.float32)
+    hi = np.array([250, 250, 100, 250, 250, 10], np.float32)
+    S = rt.Surrogate(lo, hi, n_freq=F, width=W, n_hidden=L, sigma=1.0, seed=7)
+    if first:
+        S.infer_layers(torch.as_tensor(_batch(first, 3)[0]).cuda())
+    x, t = _batch(B, 2)
+    p0 = S.params().cpu().numpy()
+    loss = torch.zeros(1, device="cuda")
+    S.train_step(torch.as_tensor(x).cuda(), torch.as_tensor(t).cuda(), 1e-3, loss)
+    g_gpu = S.grads().cpu().numpy()
+    torch.cuda.synchronize()
+    assert S.status() == 0
+    ref_loss, g_ref = R.loss_and_grads(p0, x, t, S.F, S.W, S.L, lo, hi, bf16=True)
+    assert abs(loss.item() - ref_loss) <= tol * abs(ref_loss)
+    o = 0
+    for l in range(L + 1):
+        fi, fo = (2 * F if l == 0 else W), (2 if l == L else W)
+        for n in (fi * fo, fo):
+            a, b = g_gpu[o:o + n], g_ref[o:o + n]
+            assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b) + 1e-12, (l, n)
+            o += n
+    S.close()
