@@ -673,6 +673,15 @@ __device__ __forceinline__ bool any_hit(const DevScene& s, const float4* sm, int
     return any_hit_b<C, V8>(s, sm, n_sm, o, d, tmax, ex0, ex1, cnt);
 }
 
+// Any occluder (any_hit), with the one found in `found` on the binary layout
+// (RT_NO_REF on the wide one, whose leaves have no such reference).
+template <int LY>
+__device__ __forceinline__ bool any_hit_ref(const DevScene& s, f3 o, f3 d, float tmax, int ex0, int ex1,
+                                            TravCount& cnt, int& found) {
+    if (LY == 8) return any_hit<false, 8>(s, nullptr, 0, o, d, tmax, ex0, ex1, cnt);
+    return any_hit_b<false, true, true>(s, nullptr, 0, o, d, tmax, ex0, ex1, cnt, &found);
+}
+
 // Spherical Fibonacci lattice direction of ray i of N (global frame):
 // z = 1 - (2i+1)/N, phi = 2 pi frac(i (sqrt5 - 1)/2), computed in FP64 and
 // rounded to FP32 once (Sec. II-B: directions on a Fibonacci lattice).

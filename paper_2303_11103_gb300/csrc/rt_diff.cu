@@ -88,15 +88,6 @@ __device__ __forceinline__ void pair_devices(const int32_t* rx_off, int n_tx, in
     }
 }
 
-// Any occluder (any_hit), with the one found in `found` on the binary layout
-// (RT_NO_REF on the wide one, whose leaves have no such reference).
-template <int LY>
-__device__ __forceinline__ bool any_hit_ref(const DevScene& s, f3 o, f3 d, float tmax, int ex0, int ex1,
-                                            TravCount& cnt, int& found) {
-    if (LY == 8) return any_hit<false, 8>(s, nullptr, 0, o, d, tmax, ex0, ex1, cnt);
-    return any_hit_b<false, true, true>(s, nullptr, 0, o, d, tmax, ex0, ex1, cnt, &found);
-}
-
 // D -> rx of the last (up to 32) of a warp's n2 queued candidates; the open
 // ones are paths. Called by all 32 lanes.
 template <int LY>

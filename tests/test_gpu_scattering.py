@@ -168,3 +168,34 @@ def test_negative_coefficient_scatters_nothing(tracer):
     assert np.all(np.abs(g - og) <= 2e-3 * og + 1e-3 * og.sum(axis=(1, 2), keepdims=True)), (g, og)
     gs = tracer.scattering_gain_vjp(N, np.ones((2, 1, 2), np.float32)).cpu().numpy()
     assert gs[0] == 0.0 and gs[2] == 0.0 and gs[1] > 0.0
+
+
+@pytest.mark.parametrize("N,n_rx,n_tx", [(1, 1, 1),         # one ray, one receiver
+                                         (33, 65, 2),       # a unit of one ray over, a receiver over two chunks
+                                         (700, 40, 1),      # units of 32 rays, one chunk
+                                         (60000, 33, 1)])   # whole units, the last one ragged
+def test_scattering_unit_edges(N, n_rx, n_tx):
+    """Ray and receiver counts at the edges of the work units, against the
+    oracle (tolerance: as above, a near-degenerate ray may land on either side)."""
+    tr = rt.Tracer(0, FC)
+    try:
+        sc = S.tiny_scene()
+        rng = np.random.default_rng(N)
+        tx = S.Devices(np.array([[-60.0, 0.0, 25.0], [0.0, 50.0, 10.0]], np.float32)[:n_tx],
+                       np.zeros((n_tx, 3), np.float32), S.V_ISO)
+        xy = rng.uniform(-95.0, 95.0, size=(4 * n_rx, 2))
+        xy = xy[(np.abs(xy[:, 0]) > 12.0) | (np.abs(xy[:, 1]) > 12.0)][:n_rx]
+        rx = S.Devices(np.concatenate([xy, np.full((n_rx, 1), 1.5)], 1).astype(np.float32),
+                       np.zeros((n_rx, 3), np.float32), S.V_ISO)
+        setup(tr, sc, tx, rx)
+        S_m = np.array([0.6], np.float32)
+        tr.set_scattering(S_m)
+        g = tr.scattering_gain(N).cpu().numpy()
+        osc = O.make_scene(sc)
+        for t in range(n_tx):
+            og = SC.scattering_gain(osc, sc.mat_id, S_m.astype(np.float64), FC, tx, rx, N, tx_index=t)
+            got = g[t * n_rx:(t + 1) * n_rx]
+            tol = 2e-3 * og + (1e-3 if N > 1000 else 1.0 / N) * og.sum(axis=(1, 2), keepdims=True)
+            assert np.all(np.abs(got - og) <= tol), (t, np.abs(got - og).max(), og.max())
+    finally:
+        tr.close()
