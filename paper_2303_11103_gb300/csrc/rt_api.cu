@@ -86,6 +86,8 @@ DevScene dev_scene(rt_ctx* ctx) {
     s.n_nodes = ctx->n_nodes;
     s.n_mat = ctx->n_mat;
     s.tmin = ctx->tmin;
+    s.pk = bp<float4>(ctx->pk);
+    s.pk_rho = 0.5f * ctx->extent / std::sqrt((float)std::max((ctx->n_bvh + 31) / 32, 1));
     return s;
 }
 
@@ -254,7 +256,7 @@ int rt_destroy(rt_ctx* ctx) {
         buf_free(ctx->side_counters);
         buf_free(ctx->side_status);
     }
-    for (DevBuf* b : {&ctx->nodes, &ctx->tris, &ctx->tris_o, &ctx->planes, &ctx->planes64, &ctx->mat, &ctx->mats, &ctx->tx_pos,
+    for (DevBuf* b : {&ctx->nodes, &ctx->pk, &ctx->tris, &ctx->tris_o, &ctx->planes, &ctx->planes64, &ctx->mat, &ctx->mats, &ctx->tx_pos,
                       &ctx->tx_ypr, &ctx->rx_pos, &ctx->rx_ypr, &ctx->rx_off_d, &ctx->keys, &ctx->keys_alt,
                       &ctx->vals, &ctx->vals_alt, &ctx->ray_hits, &ctx->cand_key, &ctx->cand_wit, &ctx->cand_off,
                       &ctx->cand_img, &ctx->htab_key, &ctx->htab_wit, &ctx->htab_cnt, &ctx->dop_cyc, &ctx->arr_dirs,
@@ -743,7 +745,7 @@ static std::vector<void*> graph_buffers(rt_ctx* ctx) {
     std::vector<void*> v;
     for (DevBuf* b : {&ctx->nodes, &ctx->wnodes, &ctx->tris, &ctx->tris_o, &ctx->planes, &ctx->planes64, &ctx->mat,
                       &ctx->mats, &ctx->tx_pos, &ctx->tx_ypr, &ctx->rx_pos, &ctx->rx_ypr, &ctx->rx_off_d, &ctx->perm,
-                      &ctx->dirs, &ctx->counters, &ctx->status, &ctx->scat, &ctx->scat_alpha})
+                      &ctx->dirs, &ctx->counters, &ctx->status, &ctx->scat, &ctx->scat_alpha, &ctx->pk})
         v.push_back(b->p);
     return v;
 }

@@ -895,6 +895,69 @@ float host_unord(unsigned u) {
 
 }  // namespace
 
+// Boxes for traversal by beams (layout: rt_packet.cuh): a block takes 1024
+// consecutive leaves, a warp 32 of them; the block after the last set takes
+// the header, the large triangles and the padding. Every box is widened by
+// `margin`.
+__global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tris, int n, int n_big, float margin,
+                                                   int groups, int sets, float4* __restrict__ pk) {
+    float4 *b0 = pk + 2, *b1 = b0 + 64 * (size_t)groups, *b2 = b1 + 64 * (size_t)sets;
+    float4* bb = b2 + 64 * (size_t)((sets + 31) / 32);
+    __shared__ float sb[32][6];
+    const float inf = __int_as_float(0x7f800000);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto put = [](float4* p, const float (&b)[6], int ref) {
+        p[0] = make_float4(b[0], b[1], b[2], b[3]);
+        p[1] = make_float4(b[4], b[5], __int_as_float(ref), 0.0f);
+    };
+    auto leaf = [&](int k, bool in, float (&b)[6]) {
+        for (int q = 0; q < 3; q++) {
+            b[q] = inf;
+            b[3 + q] = -inf;
+        }
+        if (!in) return;
+        const f3 v = xyz(tris[3 * (size_t)k]), e1 = xyz(tris[3 * (size_t)k + 1]), e2 = xyz(tris[3 * (size_t)k + 2]);
+        const float p[3][3] = {{v.x, v.x + e1.x, v.x + e2.x}, {v.y, v.y + e1.y, v.y + e2.y}, {v.z, v.z + e1.z, v.z + e2.z}};
+        for (int q = 0; q < 3; q++) {
+            b[q] = fminf(p[q][0], fminf(p[q][1], p[q][2])) - margin;
+            b[3 + q] = fmaxf(p[q][0], fmaxf(p[q][1], p[q][2])) + margin;
+        }
+    };
+    float b[6];
+    if ((int)blockIdx.x == sets) {
+        if (threadIdx.x == 0) *reinterpret_cast<int4*>(pk) = make_int4(groups, sets, (n_big + 31) / 32 * 32, 0);
+        for (int k = threadIdx.x; k < (n_big + 31) / 32 * 32; k += blockDim.x) {
+            leaf(n + k, k < n_big, b);
+            put(bb + 2 * (size_t)k, b, n + k);
+        }
+        for (int k = sets + threadIdx.x; k < (sets + 31) / 32 * 32; k += blockDim.x) {
+            leaf(0, false, b);
+            put(b2 + 2 * (size_t)k, b, 0);
+        }
+        return;
+    }
+    const int g = 32 * blockIdx.x + w, k = 32 * g + lane;
+    leaf(k, k < n, b);
+    if (g < groups) put(b0 + 2 * (size_t)k, b, k);
+    auto reduce = [&]() {
+        for (int q = 0; q < 3; q++)
+            for (int o = 16; o > 0; o >>= 1) {
+                b[q] = fminf(b[q], __shfl_xor_sync(0xffffffffu, b[q], o));
+                b[3 + q] = fmaxf(b[3 + q], __shfl_xor_sync(0xffffffffu, b[3 + q], o));
+            }
+    };
+    reduce();
+    if (lane == 0) {
+        put(b1 + 2 * (size_t)g, b, 0);
+        for (int q = 0; q < 6; q++) sb[w][q] = b[q];
+    }
+    __syncthreads();
+    if (w != 0) return;
+    for (int q = 0; q < 6; q++) b[q] = sb[lane][q];
+    reduce();
+    if (lane == 0) put(b2 + 2 * (size_t)blockIdx.x, b, 0);
+}
+
 int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     const int T = (int)n_tris;
     cudaStream_t st = ctx->stream;
@@ -1151,6 +1214,13 @@ int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     // leaf records in sorted order: the hierarchy's leaves, then the large triangles
     prof_begin(ctx, "k_leaf_tris");
     k_leaf_tris<<<gT, B, 0, st>>>(T, leaf_tri, bp<float4>(ctx->tris_o), bp<float4>(ctx->tris));
+    prof_end(ctx);
+    RT_TRY(cudaGetLastError());
+    const int groups = (n + 31) / 32, sets = (groups + 31) / 32;
+    RT_TRY(buf_reserve(ctx->pk, 32 * (1 + 32 * ((size_t)groups + sets + (sets + 31) / 32 + (n_big + 31) / 32))));
+    prof_begin(ctx, "k_pk_boxes");
+    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), n, (int)n_big, 4e-6f * ext, groups, sets,
+                                          bp<float4>(ctx->pk));
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
     ctx->n_wnodes = 0;

@@ -73,6 +73,8 @@ struct DevScene {
     const float2* __restrict__ mats;    // [M] eps_r, sigma
     int n_tris, n_nodes, n_mat, n_big;
     float tmin;                         // self-intersection offset (metres)
+    const float4* __restrict__ pk;      // boxes for traversal by beams (rt_packet.cuh)
+    float pk_rho;                       // spread of a beam's origins (metres)
 };
 
 __device__ __forceinline__ float4 ldg4(const float4* p) { return __ldg(p); }
@@ -326,11 +328,12 @@ __device__ __forceinline__ void flush_counts(TravCount& c, unsigned long long* c
 // The hierarchy is checked at build time to be a tree whose children have
 // larger indices than their parent (level order), with depth below
 // RT_STACK, so the loop visits each node at most once and the stack cannot
-// overflow. C: count node / triangle records and queries in cnt.
-template <bool C, bool V8>
+// overflow. C: count node / triangle records and queries in cnt. TO: hits
+// before t_out's value on entry, and with `any` set the first one found.
+template <bool C, bool V8, bool TO = false>
 __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm, int n_sm, f3 o, f3 d,
-                                             int exclude, float& t_out, TravCount& cnt) {
-    t_out = __int_as_float(0x7f800000);
+                                             int exclude, float& t_out, TravCount& cnt, bool any = false) {
+    if (!TO) t_out = __int_as_float(0x7f800000);
     if (C) cnt.queries++;
     if (s.n_tris == 0) return -1;
     f3 inv = safe_inv(d);
@@ -338,7 +341,7 @@ __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm
     int stack[RT_STACK];
     int sp = 0;
     int node = 0;
-    float tb = __int_as_float(0x7f800000);
+    float tb = t_out;
     int best = -1;
     const float tmin = s.tmin;
     // large triangles first: a hit there also bounds the traversal below
@@ -407,13 +410,13 @@ __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm
             if (sp == 0) break;
             node = stack[--sp];
         }
+        if (TO && any && best >= 0) return best;
     }
-    t_out = tb;
+    if (!(TO && any)) t_out = tb;
     return best;
 }
 
-// A triangle as the traversal reaches it: 2 * node + child for a leaf of the
-// binary hierarchy, -2 - k for large triangle k, RT_NO_REF for none.
+// No occluder, where any_hit_b and ref_hit name one by its index in s.tris.
 #define RT_NO_REF (-1)
 
 // Any occluder on the open segment (tmin, tmax) along o + t d (d unit),
@@ -437,7 +440,7 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
         if (id != ex0 && id != ex1) {
             float t = tri_hit(r0, r1, r2, o, d);
             if (t > tmin && t < tmax) {
-                if (REF) *ref = -2 - k;
+                if (REF) *ref = (int)((s.big - s.tris) / 3) + k;
                 return true;
             }
         }
@@ -460,7 +463,7 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
             if (id != ex0 && id != ex1) {
                 float t = tri_hit(r0, r1, r2, o, d);
                 if (t > tmin && t < tmax) {
-                    if (REF) *ref = 2 * node + 0;
+                    if (REF) *ref = ~c0;
                     return true;
                 }
             }
@@ -474,7 +477,7 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
             if (id != ex0 && id != ex1) {
                 float t = tri_hit(r0, r1, r2, o, d);
                 if (t > tmin && t < tmax) {
-                    if (REF) *ref = 2 * node + 1;
+                    if (REF) *ref = ~c1;
                     return true;
                 }
             }
@@ -495,27 +498,12 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
     return false;
 }
 
-// Whether the triangle `ref` (from an earlier any_hit_b) occludes this segment:
-// one box test and one triangle test instead of a traversal. True exactly
-// where the traversal would report this triangle as a hit: it reaches a leaf
-// whose own box is hit, since every ancestor's planes enclose the leaf's and
-// a plane's distance (one FMA, rounded once) is monotone in the plane.
+// Whether the triangle `ref` (from an earlier any_hit_b) occludes this
+// segment: one triangle test instead of a traversal. The traversal would find
+// it too: a leaf's box is padded beyond what rounding can shift a hit.
 __device__ __forceinline__ bool ref_hit(const DevScene& s, int ref, f3 o, f3 d, float tmax, int ex0, int ex1) {
     if (ref == RT_NO_REF) return false;
-    const float4* tp;
-    if (ref < 0) {
-        tp = s.big + 3 * (size_t)(-2 - ref);
-    } else {
-        const f3 inv = safe_inv(d);
-        const f3 oi = {o.x * inv.x, o.y * inv.y, o.z * inv.z};
-        float4 a, b, c, e;
-        load_node<true>(octant_nodes(s, inv) + 4 * (size_t)(ref >> 1), a, b, c, e);
-        float tn0, tf0, tn1, tf1;
-        box_pair(a, b, c, pair_ray(inv, oi), s.tmin, tmax, tn0, tf0, tn1, tf1);
-        const bool second = ref & 1;
-        if (!((second ? tn1 : tn0) <= (second ? tf1 : tf0))) return false;
-        tp = s.tris + 3 * (size_t)(~__float_as_int(second ? e.y : e.x));
-    }
+    const float4* tp = s.tris + 3 * (size_t)ref;
     const float4 r0 = ldg4(tp), r1 = ldg4(tp + 1), r2 = ldg4(tp + 2);
     const int id = __float_as_int(r0.w);
     if (id == ex0 || id == ex1) return false;

@@ -46,6 +46,7 @@ struct rt_ctx {
     DevBuf wnodes;        // 8-wide layout [n_wnodes * RT_WN_F4] (when bvh_width == 8)
     int n_wnodes = 0;
     DevBuf planes64;   // [T*3] double2: FP64 unit normal and first vertex per triangle (original order)
+    DevBuf pk;                 // boxes for traversal by beams (rt_packet.cuh)
 
     // devices
     int n_tx = 0, n_rx = 0;

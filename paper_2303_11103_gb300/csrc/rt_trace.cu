@@ -11,23 +11,40 @@
 // levels are staged in shared memory once per block.
 #include "rt_field.cuh"
 #include "rt_internal.h"
+#include "rt_packet.cuh"
 
 namespace {
 
 // -------------------------------------------------------------- ray ordering
-// Key = 2D Morton code of (z, phi) of the lattice direction quantised to
-// 2^12 x 2^12 cells: rays whose order is close point in close directions.
+// Key = place of the lattice direction along Hilbert curves over (phi, z),
+// three squares of 120 degrees by 2 (equal areas, nearly square in angle) of
+// 2^11 x 2^11 cells each: any run of rays in this order points into one patch
+// of directions (a Z-order curve jumps, and splits such a run in two).
 __global__ void k_perm_keys(long long N, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     f3 d = fib_dir(N, i);
     float u = fminf(fmaxf((d.z + 1.0f) * 0.5f, 0.0f), 0.99999f);
     float v = (atan2f(d.y, d.x) + RT_PI_F) * (0.5f / RT_PI_F);
-    v = fminf(fmaxf(v, 0.0f), 0.99999f);
-    unsigned a = (unsigned)(u * 4096.0f), b = (unsigned)(v * 4096.0f);
-    unsigned long long code = 0;
-    for (int k = 0; k < 12; k++) code |= (unsigned long long)(((a >> k) & 1u) << (2 * k + 1)) |
-                                        (unsigned long long)(((b >> k) & 1u) << (2 * k));
+    v = 3.0f * fminf(fmaxf(v, 0.0f), 0.99999f);
+    const unsigned third = (unsigned)v;
+    unsigned x = (unsigned)((v - (float)third) * 2048.0f), y = (unsigned)(u * 2048.0f);
+    unsigned code = third;
+    // quadrant by quadrant from the top: (0,0), (0,1), (1,1), (1,0), the curve
+    // inside the first mirrored in the diagonal and in the last in the other one
+    for (int k = 10; k >= 0; k--) {
+        const unsigned rx = (x >> k) & 1u, ry = (y >> k) & 1u;
+        code = (code << 2) | ((3u * rx) ^ ry);
+        if (ry == 0) {
+            if (rx) {
+                x = ~x;
+                y = ~y;
+            }
+            const unsigned t = x;
+            x = y;
+            y = t;
+        }
+    }
     keys[i] = code;
     vals[i] = (uint32_t)i;
 }
@@ -64,7 +81,18 @@ __device__ __forceinline__ void stage_nodes(const TraceCommon& c, float4* sm) {
     __syncthreads();
 }
 
-// Warp-level ray fetch: refill dead lanes from the warp's chunk. Returns the
+// a / b for 0 <= a, 0 < b: in 32 bits where both fit, about a fifth of the
+// 64-bit division's instructions.
+__device__ __forceinline__ long long div_ll(long long a, long long b) {
+    if (((a | b) >> 32) == 0) return (unsigned)a / (unsigned)b;
+    return a / b;
+}
+
+// Warp-level ray fetch: when all lanes are dead, the next rays of the warp's
+// chunk. Lanes whose rays ended early wait for the others: the rays of a refill
+// start side by side and mostly hit the same surfaces, which a ray of another
+// patch among them breaks (64-transmitter map: 121 ms, against 151 when every
+// dead lane was refilled at once, both ray by ray). Returns the
 // global ray slot (tx * N + lattice index) for a refilled lane, -1 otherwise.
 struct WarpFeed {
     long long next = 0, end = 0;
@@ -75,7 +103,7 @@ struct WarpFeed {
         const unsigned full = 0xffffffffu;
         unsigned dead = __ballot_sync(full, !alive);
         long long slot = -1;
-        if (dead == 0 || exhausted) return slot;
+        if (dead != full || exhausted) return slot;
         if (next >= end) {
             // a warp with a refill quota stops after it (its block then ends
             // and frees its SM slot for other work)
@@ -98,8 +126,8 @@ struct WarpFeed {
         int take = (int)min((long long)need, end - next);
         int r = __popc(dead & lanemask_lt());
         if (!alive && r < take) {
-            long long q = next + r;
-            long long tx = q / c.count, k = q - tx * c.count;
+            const long long q = next + r;
+            const long long tx = div_ll(q, c.count), k = q - tx * c.count;
             long long i = c.perm ? (long long)c.perm[k] : c.first + k;
             slot = tx * c.N + i;
             k_out = k;
@@ -127,7 +155,8 @@ struct SbrParams {
     int32_t* hits;                 // [total*D] or null
 };
 
-template <bool C, int L>
+// B: rays traced as beams (rt_packet.cuh)
+template <bool C, int L, bool B = false>
 __global__ void __launch_bounds__(256) k_sbr(SbrParams p) {
     extern __shared__ float4 sm[];
     stage_nodes(p.c, sm);
@@ -143,7 +172,7 @@ __global__ void __launch_bounds__(256) k_sbr(SbrParams p) {
         long long s = feed.refill(p.c, alive, kd);
         if (s >= 0) {
             slot = s;
-            long long tx = s / p.c.N, i = s - tx * p.c.N;
+            const long long tx = div_ll(s, p.c.N), i = s - tx * p.c.N;
             o = mk(p.c.tx_pos[3 * tx], p.c.tx_pos[3 * tx + 1], p.c.tx_pos[3 * tx + 2]);
             d = ray_dir(p.c, kd, i);
             last = -1;
@@ -158,9 +187,11 @@ __global__ void __launch_bounds__(256) k_sbr(SbrParams p) {
         bool emit = false;
         uint64_t ekey = 0;
         uint32_t epos = 0;
+        float t = __int_as_float(0x7f800000);
+        int id = -1;
+        if (B) warp_trace(p.c.s, alive, false, o, d, last, t, id);
+        else if (alive) id = closest_hit<C, L, false>(p.c.s, sm, p.c.n_sm, o, d, last, t, cnt);
         if (alive) {
-            float t;
-            int id = closest_hit<C, L, false>(p.c.s, sm, p.c.n_sm, o, d, last, t, cnt);
             if (id < 0) {
                 alive = false;
             } else {
@@ -262,12 +293,28 @@ __device__ __forceinline__ long long cov_segment(const CovParams& p, const float
     return any_hit<C, L>(p.c.s, sm, p.c.n_sm, o, d, up, last, last, cnt_pl) ? -1 : cell;
 }
 
+// cov_segment for all lanes of a warp (alive: those that hold a ray); called
+// by all 32 lanes.
+template <bool C, int L, bool B>
+__device__ __forceinline__ long long cov_segment_warp(const CovParams& p, const float4* sm, bool alive, int tx, f3 o,
+                                                      f3 d, int last, bool more, int& id, float& t, TravCount& cnt,
+                                                      TravCount& cnt_pl) {
+    id = -1;
+    if (!B) return alive ? cov_segment<C, L>(p, sm, tx, o, d, last, more, id, t, cnt, cnt_pl) : -1;
+    float sc = 0.0f;
+    const long long cell = alive ? plane_cell(p, tx, o, d, sc) : -1;
+    // t <= sc  <=>  t < the next float above sc (sc is finite here)
+    t = more ? __int_as_float(0x7f800000) : nextafterf(sc, __int_as_float(0x7f800000));
+    warp_trace(p.c.s, alive && (more || cell >= 0), !more, o, d, last, t, id);
+    return cell >= 0 && (id < 0 || (more && sc < t)) ? cell : -1;
+}
+
 // Transmitter rotations a coverage block keeps in shared memory (more
 // transmitters: computed per ray).
 #define RT_ROT_CACHE 64
 
-template <bool C, int L>
-__global__ void __launch_bounds__(256) k_coverage(CovParams p) {
+template <bool C, int L, bool B = false>
+__global__ void __launch_bounds__(256, 4) k_coverage(CovParams p) {
     extern __shared__ float4 sm[];
     // each transmitter's rotation once per block instead of once per ray
     // (the same function, so the same values)
@@ -293,7 +340,7 @@ __global__ void __launch_bounds__(256) k_coverage(CovParams p) {
         long long kd = 0;
         long long s = feed.refill(p.c, alive, kd);
         if (s >= 0) {
-            long long t64 = s / p.c.N, i = s - t64 * p.c.N;
+            const long long t64 = div_ll(s, p.c.N), i = s - t64 * p.c.N;
             tx = (int)t64;
             o = mk(p.c.tx_pos[3 * tx], p.c.tx_pos[3 * tx + 1], p.c.tx_pos[3 * tx + 2]);
             d = ray_dir(p.c, kd, i);
@@ -315,11 +362,11 @@ __global__ void __launch_bounds__(256) k_coverage(CovParams p) {
             if (feed.exhausted) break;
             continue;
         }
+        float t;
+        int id;
+        const bool more = depth < p.D;
+        const long long cell = cov_segment_warp<C, L, B>(p, sm, alive, tx, o, d, last, more, id, t, cnt, cnt_pl);
         if (alive) {
-            float t;
-            int id;
-            const bool more = depth < p.D;
-            const long long cell = cov_segment<C, L>(p, sm, tx, o, d, last, more, id, t, cnt, cnt_pl);
             if (cell >= 0) {
                 V3<float> F = antenna_vec<float>(p.rxa.kind, zeta_r, Rr, V3<float>{-d.x, -d.y, -d.z});
                 float re = F.x * E[0].re + F.y * E[1].re + F.z * E[2].re;
@@ -366,8 +413,11 @@ struct CovVjpParams {
 
 __device__ __forceinline__ void flush_ypr(float* g, int tx, float (&acc)[3]) {
     const unsigned full = 0xffffffffu;
-    const int t0 = __shfl_sync(full, tx, 0);
-    if (__all_sync(full, tx == t0)) {
+    // lanes without a transmitter (tx -1) have nothing to add
+    const unsigned has = __ballot_sync(full, tx >= 0);
+    const int t0 = __shfl_sync(full, tx, has ? __ffs(has) - 1 : 0);
+    if (tx < 0) acc[0] = acc[1] = acc[2] = 0.0f;
+    if (__all_sync(full, tx == t0 || tx < 0)) {
         for (int k = 0; k < 3; k++) {
             float v = acc[k];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
@@ -380,7 +430,7 @@ __device__ __forceinline__ void flush_ypr(float* g, int tx, float (&acc)[3]) {
     acc[0] = acc[1] = acc[2] = 0.0f;
 }
 
-template <int L>
+template <int L, bool B = false>
 __global__ void __launch_bounds__(256) k_coverage_vjp(CovVjpParams q) {
     extern __shared__ float4 sm[];
     const CovParams& p = q.p;
@@ -399,7 +449,7 @@ __global__ void __launch_bounds__(256) k_coverage_vjp(CovVjpParams q) {
         long long kd = 0;
         long long s = feed.refill(p.c, alive, kd);
         // a lane moving to another transmitter flushes its accumulators first
-        const int next_tx = s >= 0 ? (int)(s / p.c.N) : tx;
+        const int next_tx = s >= 0 ? (int)div_ll(s, p.c.N) : tx;
         if (__any_sync(0xffffffffu, next_tx != tx && tx >= 0)) {
             int ftx = (next_tx != tx) ? tx : -1;
             float keep[3] = {acc[0], acc[1], acc[2]};
@@ -430,11 +480,11 @@ __global__ void __launch_bounds__(256) k_coverage_vjp(CovVjpParams q) {
             if (feed.exhausted) break;
             continue;
         }
+        float t;
+        int id;
+        const bool more = depth < p.D;
+        const long long cell = cov_segment_warp<false, L, B>(p, sm, alive, tx, o, d, last, more, id, t, cnt, cnt);
         if (alive) {
-            float t;
-            int id;
-            const bool more = depth < p.D;
-            const long long cell = cov_segment<false, L>(p, sm, tx, o, d, last, more, id, t, cnt, cnt);
             if (cell >= 0) {
                 const float g = q.grad_gain[cell];
                 if (g != 0.0f) {
@@ -481,14 +531,18 @@ int trace_grid(rt_ctx* ctx, const void* kernel, size_t smem) {
     return per_sm * ctx->num_sms;
 }
 
-// Rays per warp refill: the tuned value, else 32 (one ray per lane). Larger
-// refills cut the counter atomics but lengthen the launch's tail and keep a
-// warp on one patch of directions; on the 64-transmitter coverage map (6.4e8
-// rays) 32 ran 2.1x faster than 1024.
+// Rays per warp refill: the tuned value, else 32 (one ray per lane), or fewer
+// (down to 4) while that leaves warps of the grid without rays: a warp's rays
+// are then closer together and its longest one shorter. Larger refills cut the
+// counter atomics but lengthen the launch's tail and keep a warp on one patch
+// of directions; on the 64-transmitter coverage map (6.4e8 rays) 32 ran 2.1x
+// faster than 1024.
 int pick_chunk(rt_ctx* ctx, long long total, int grid) {
-    (void)total;
-    (void)grid;
-    return ctx->warp_chunk > 0 ? ctx->warp_chunk : 32;
+    if (ctx->warp_chunk > 0) return ctx->warp_chunk;
+    const long long warps = (long long)grid * (ctx->trace_block / 32);
+    int chunk = 32;
+    while (chunk > 4 && total < chunk * warps) chunk /= 2;
+    return chunk;
 }
 
 }  // namespace
@@ -563,6 +617,20 @@ static TraceCommon make_common(rt_ctx* ctx, int64_t N, int64_t first, int64_t co
     return c;
 }
 
+// Whether a trace takes its rays as beams: on the binary layout, with no
+// traversal counts asked for, in the direction-coherent order, and from
+// PK_DENSITY rays per transmitter and triangle on. A warp's 32 rays then span
+// less than about a sixth of the spacing of the leaf groups at a quarter of the
+// scene's extent; wider beams meet more triangles than a ray's own traversal
+// does. City of 4802 triangles, 32 transmitters, depth 3, beams against single
+// rays: 2e4 rays each 401 / 238 us, 6e4 528 / 433, 2e5 957 / 1035; 4
+// transmitters of 1e6, map, 861 / 972; 770 triangles: 2e4 214 / 235, 6e4
+// 300 / 539.
+constexpr long long PK_DENSITY = 40;
+static bool use_beams(const rt_ctx* ctx, const TraceCommon& c) {
+    return !wide_layout(ctx) && !ctx->count_work && c.perm && ctx->n_tris > 0 && c.N >= PK_DENSITY * ctx->n_tris;
+}
+
 // Shoot and bounce: appends every hit's candidate key with its position
 // (tx*N + i)*D + depth; the key count goes to counter slot RT_CNT_KEYS.
 int launch_sbr(rt_ctx* ctx, int64_t N, int D, uint64_t* keys, uint32_t* vals, int32_t* hits) {
@@ -581,6 +649,7 @@ int launch_sbr(rt_ctx* ctx, int64_t N, int D, uint64_t* keys, uint32_t* vals, in
     size_t smem = staged_bytes(ctx);
     auto kern = wide_layout(ctx) ? (ctx->count_work ? k_sbr<true, 8> : k_sbr<false, 8>)
                                  : (ctx->count_work ? k_sbr<true, 2> : k_sbr<false, 2>);
+    if (use_beams(ctx, p.c)) kern = k_sbr<false, 2, true>;
     RT_TRY(ensure_smem_attr((const void*)kern, smem));
     RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), ctx->stream));
     RT_TRY(cudaMemsetAsync(p.n_keys, 0, sizeof(unsigned long long), ctx->stream));
@@ -625,6 +694,7 @@ int launch_coverage(rt_ctx* ctx, const rt_grid* g, int D, int64_t N, int64_t fir
     size_t smem = staged_bytes(ctx);
     auto kern = wide_layout(ctx) ? (ctx->count_work ? k_coverage<true, 8> : k_coverage<false, 8>)
                                  : (ctx->count_work ? k_coverage<true, 2> : k_coverage<false, 2>);
+    if (use_beams(ctx, p.c)) kern = k_coverage<false, 2, true>;
     RT_TRY(ensure_smem_attr((const void*)kern, smem));
     RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), ctx->stream));
     int grid = trace_grid(ctx, (const void*)kern, smem);
@@ -674,7 +744,7 @@ int launch_coverage_vjp(rt_ctx* ctx, const rt_grid* g, int D, int64_t N, int tx_
     q.grad_ypr = grad_ypr;
     RT_TRY(cudaMemsetAsync(grad_ypr, 0, sizeof(float) * 3 * (size_t)ctx->n_tx, ctx->stream));
     size_t smem = staged_bytes(ctx);
-    auto kern = wide_layout(ctx) ? k_coverage_vjp<8> : k_coverage_vjp<2>;
+    auto kern = wide_layout(ctx) ? k_coverage_vjp<8> : use_beams(ctx, p.c) ? k_coverage_vjp<2, true> : k_coverage_vjp<2>;
     RT_TRY(ensure_smem_attr((const void*)kern, smem));
     RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), ctx->stream));
     int grid = trace_grid(ctx, (const void*)kern, smem);
