@@ -34,6 +34,7 @@
 
 #include "rt_field.cuh"
 #include "rt_internal.h"
+#include "rt_packet.cuh"
 
 namespace {
 
@@ -67,6 +68,7 @@ struct DiffFind {
     int tiles, runs;         // receiver tiles of 32 (of the largest receiver set), runs of DF_RUN tiles
     CellGrid grid;           // receivers at cell centres when grid.nx > 0
     unsigned long long* count;
+    unsigned long long* work;   // units taken (cleared with the count)
     unsigned long long cap;
     uint64_t* keys;          // pair << 32 | wedge
     float4* pts;             // diffraction points
@@ -92,7 +94,7 @@ __device__ __forceinline__ void pair_devices(const int32_t* rx_off, int n_tx, in
 // ones are paths. Called by all 32 lanes.
 template <int LY>
 __device__ __forceinline__ void diff_tail(const DiffFind& p, const int* qr, const float* qt, int& n2, int t, int wi,
-                                          f3 A, f3 e, int f0, int f1, int& ref2, TravCount& cnt) {
+                                          f3 A, f3 e, int f0, int f1, int& ref2) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int take = min(n2, 32);
@@ -100,14 +102,15 @@ __device__ __forceinline__ void diff_tail(const DiffFind& p, const int* qr, cons
     bool open = false;
     int found = RT_NO_REF, r = 0;
     f3 D = mk(0.0f, 0.0f, 0.0f);
+    f3 rx = D;
     if (lane < take) {
         r = qr[n2 + lane];
         D = A + e * qt[n2 + lane];
-        const f3 rx = p.grid.nx > 0 ? cell_centre(p.grid, r) : mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
-        const f3 d = rx - D;
-        const float L = sqrtf(dot(d, d));
-        open = !any_hit_ref<LY>(p.s, D, d * (1.0f / L), L - p.s.tmin, f0, f1, cnt, found);
+        rx = p.grid.nx > 0 ? cell_centre(p.grid, r) : mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
     }
+    const f3 d = rx - D;
+    const float L = sqrtf(dot(d, d));
+    open = !warp_segments<LY>(p.s, lane < take, D, rx, d * (1.0f / L), L - p.s.tmin, f0, f1, found) && lane < take;
     const unsigned fm = __ballot_sync(full, found != RT_NO_REF);
     if (fm) ref2 = __shfl_sync(full, found, 31 - __clz(fm));
     const unsigned m = __ballot_sync(full, open);
@@ -131,6 +134,27 @@ __device__ __forceinline__ void diff_tail(const DiffFind& p, const int* qr, cons
 constexpr int DF_RUN = 64;
 constexpr int DF_TX = 8, DF_TY = 4;
 constexpr int DF_Q = 64;   // entries of a warp's queues
+constexpr int DF_UNITS = 4;   // units a warp takes at a time
+
+// Whether some cell of a grid tile may have its Keller point on the edge
+// (0 < t < len): t = ts + (tr - ts) rs / (rs + rr) for the extremes of tr
+// (place along the edge) and rr (distance from it) over the tile, which lies
+// within `rad` of its centre, widened by far more than rounding.
+__device__ __forceinline__ bool tile_reached(const CellGrid& g, int tile, int tiles_y, f3 A, f3 e, float len, float ts,
+                                             float rs) {
+    const int cx = tile / tiles_y, cy = tile - cx * tiles_y;
+    const f3 c = mk(g.x0 + ((float)(cx * DF_TX) + 0.5f * DF_TX) * g.cell, g.y0 + ((float)(cy * DF_TY) + 0.5f * DF_TY) * g.cell, g.h);
+    const float rad = 0.5f * sqrtf((float)(DF_TX * DF_TX + DF_TY * DF_TY)) * g.cell;
+    const f3 v = c - A;
+    const float tr = dot(v, e) - ts;
+    const f3 pr = v - e * (tr + ts);
+    const float rr = sqrtf(dot(pr, pr));
+    const float slack = 1e-4f * (fabsf(ts) + fabsf(tr) + rr + rs + rad);
+    const float w0 = rs / (rs + rr + rad), w1 = rs / fmaxf(rs + fmaxf(rr - rad, 0.0f), 1e-30f);
+    const float lo = tr - rad, hi = tr + rad;
+    const float tmin = ts + fminf(lo * w0, lo * w1), tmax = ts + fmaxf(hi * w0, hi * w1);
+    return !(tmax < -slack || tmin > len + slack);
+}
 
 // Every (transmitter, wedge, receiver): Keller point, exterior test, two
 // segment occlusion tests; valid paths are appended (order fixed afterwards
@@ -142,11 +166,19 @@ constexpr int DF_Q = 64;   // entries of a warp's queues
 // triangle instead of a traversal); the candidates it does not block are
 // queued, so that the traversals run with all 32 lanes.
 //
+// The queued segments of a warp lie side by side (one wedge, neighbouring cells)
+// and go through the scene as a beam (warp_segments). Tiles of a map whose cells
+// all have their Keller point off the edge are left out, 32 of them tested at a
+// time. Units are handed out DF_UNITS at a time: dealt in turn they left some
+// SMs with twice the others' work.
+//
 // Bound by the candidates' own arithmetic and by the segments no kept
 // occluder answers. City map of 500 x 500 cells x 4800 wedges (1.2e9
-// candidates): 73.3 ms with one thread per (receiver, wedge) in wedge order
-// (7.6 of 32 lanes active, the wedge reloaded and its sincos and transmitter
-// side recomputed per candidate), 12.6 ms now.
+// candidates), mean of six sites: 4.1 ms; 73 to 87 ms with one thread per
+// (receiver, wedge) in wedge order (7.6 of 32 lanes active, the wedge reloaded
+// and its sincos and transmitter side recomputed per candidate). On the way, at
+// one site: 12.8 ms a warp a wedge, 9.8 segments as beams, 6.3 tiles left out,
+// then (10.8 at the worst site) units handed out.
 template <int LY>
 __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
     __shared__ int q1r[4][DF_Q], q2r[4][DF_Q];
@@ -154,13 +186,20 @@ __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
     const unsigned full = 0xffffffffu, lt = lanemask_lt();
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int64_t units = (int64_t)p.n_tx * p.runs * p.n_w;
-    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
     const bool map = p.grid.nx > 0;
     const int tiles_y = (p.grid.ny + DF_TY - 1) / DF_TY;
-    TravCount cnt;
-    for (int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + wp; u < units; u += step) {
+    int64_t u = 0, u_end = 0;   // this warp's units
+    while (true) {
+        if (u == u_end) {
+            unsigned long long b = 0;
+            if (lane == 0) b = atomicAdd(p.work, (unsigned long long)DF_UNITS);
+            u = (int64_t)__shfl_sync(full, b, 0);
+            if (u >= units) break;
+            u_end = min(u + DF_UNITS, units);
+        }
         const int64_t tr_ = u / p.n_w;
         const int wi = (int)(u - tr_ * p.n_w);
+        u++;
         const int t = (int)(tr_ / p.runs), run = (int)(tr_ - (int64_t)t * p.runs);
         const int r0 = p.rx_off ? p.rx_off[t] : 0;
         const int R = p.rx_off ? p.rx_off[t + 1] - r0 : p.n_rx;
@@ -178,8 +217,19 @@ __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
         int ref1 = RT_NO_REF, ref2 = RT_NO_REF;   // last occluders of tx -> D and D -> rx
         int n1 = 0, n2 = 0;                       // queued candidates (warp-uniform)
         const int tile_end = min(p.tiles, (run + 1) * DF_RUN);
-        for (int tile = run * DF_RUN; tile <= tile_end; tile++) {
-            const bool last = tile == tile_end;   // one more turn empties the queues
+        int next = run * DF_RUN;       // tiles not yet looked at, 32 at a time
+        int base = next;
+        unsigned todo = 0;             // tiles base + k that may have a path
+        while (true) {
+            while (todo == 0 && next < tile_end) {
+                base = next;
+                next += 32;
+                todo = __ballot_sync(full, base + lane < tile_end &&
+                                               (!map || tile_reached(p.grid, base + lane, tiles_y, A, e, w.a.w, ts, rs)));
+            }
+            const bool last = todo == 0;   // one more turn empties the queues
+            const int tile = base + __ffs(todo) - 1;
+            todo &= todo - 1;
             bool open1 = false;
             int r = 0;
             float tpar = 0.0f;
@@ -231,13 +281,17 @@ __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
                 n1 -= take;
                 bool open2 = false;
                 int found = RT_NO_REF;
+                f3 D = A;
                 if (lane < take) {
                     r = q1r[wp][n1 + lane];
                     tpar = q1t[wp][n1 + lane];
-                    const f3 D = A + e * tpar;
+                    D = A + e * tpar;
+                }
+                {
                     f3 d = D - tx;
                     float L = sqrtf(dot(d, d));
-                    open2 = !any_hit_ref<LY>(p.s, tx, d * (1.0f / L), L - p.s.tmin, f0, f1, cnt, found);
+                    open2 = !warp_segments<LY>(p.s, lane < take, tx, D, d * (1.0f / L), L - p.s.tmin, f0, f1, found) &&
+                            lane < take;
                     if (open2) {
                         const f3 rx = map ? cell_centre(p.grid, r) : mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
                         d = rx - D;
@@ -256,11 +310,12 @@ __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
                 n2 += __popc(m2);
                 __syncwarp();
                 if (n2 >= 32 || (last && n1 == 0 && n2 > 0)) {
-                    diff_tail<LY>(p, q2r[wp], q2t[wp], n2, t, wi, A, e, f0, f1, ref2, cnt);
+                    diff_tail<LY>(p, q2r[wp], q2t[wp], n2, t, wi, A, e, f0, f1, ref2);
                 }
             }
-            if (last)
-                while (n2 > 0) diff_tail<LY>(p, q2r[wp], q2t[wp], n2, t, wi, A, e, f0, f1, ref2, cnt);
+            if (!last) continue;
+            while (n2 > 0) diff_tail<LY>(p, q2r[wp], q2t[wp], n2, t, wi, A, e, f0, f1, ref2);
+            break;
         }
     }
 }
@@ -591,8 +646,9 @@ int diffraction_impl(rt_ctx* ctx, int64_t* n_out) {
     for (int attempt = 0; attempt < 2; attempt++) {
         RT_TRY(buf_reserve(ctx->dpath_raw_key, sizeof(uint64_t) * cap));
         RT_TRY(buf_reserve(ctx->dpath_raw_pt, sizeof(float4) * cap));
-        RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), st));
+        RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, 2 * sizeof(unsigned long long), st));
         p.count = bp<unsigned long long>(ctx->counters);
+        p.work = p.count + 1;
         p.cap = cap;
         p.keys = bp<uint64_t>(ctx->dpath_raw_key);
         p.pts = bp<float4>(ctx->dpath_raw_pt);
@@ -740,8 +796,9 @@ int diffraction_map_impl(rt_ctx* ctx, const rt_grid* g, int tx_port, float* gain
     for (int attempt = 0; attempt < 2; attempt++) {
         RT_TRY(buf_reserve(ctx->dmap_key, sizeof(uint64_t) * cap));
         RT_TRY(buf_reserve(ctx->dmap_pt, sizeof(float4) * cap));
-        RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), st));
+        RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, 2 * sizeof(unsigned long long), st));
         p.count = bp<unsigned long long>(ctx->counters);
+        p.work = p.count + 1;
         p.cap = cap;
         p.keys = bp<uint64_t>(ctx->dmap_key);
         p.pts = bp<float4>(ctx->dmap_pt);
