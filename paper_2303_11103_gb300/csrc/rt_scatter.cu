@@ -86,11 +86,11 @@ struct ScatHits {
 
 // Any occluder between a queued (hit, receiver) pair, then its contribution:
 // lane < take handles entry n + lane. Called by all 32 lanes; the occluder
-// found last goes to ref.
+// found last goes to ref0, the one before it to ref1.
 template <bool VJP, int LY>
 __device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHits& h, const int* qr,
-                                              const uint16_t* qh, int n, int take, int t, float* sgrad, int& ref,
-                                              TravCount& cnt) {
+                                              const uint16_t* qh, int n, int take, int t, float* sgrad, int& ref0,
+                                              int& ref1, TravCount& cnt) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     int r = -1, found = RT_NO_REF, m = 0;
@@ -124,7 +124,11 @@ __device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHit
         }
     }
     const unsigned fm = __ballot_sync(full, found != RT_NO_REF);
-    if (fm) ref = __shfl_sync(full, found, 31 - __clz(fm));
+    const int last = fm ? __shfl_sync(full, found, 31 - __clz(fm)) : ref0;
+    if (last != ref0) {
+        ref1 = ref0;
+        ref0 = last;
+    }
     unsigned open = __ballot_sync(full, w != 0.0f);
     const long long pair = p.rx_off ? (long long)r : (long long)t * p.n_rx + r;
     float acc = 0.0f;
@@ -164,14 +168,16 @@ __device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHit
 // direction-coherent order of the tracing kernels, so the hits of a block lie
 // near each other) and the hits that scatter are packed in shared memory; then
 // each warp takes one receiver at a time against all of them, a lane per hit.
-// The occluder that last blocked a pair of this warp is tried first (ref_hit:
-// one box and one triangle instead of a traversal), and what it does not block
-// is queued, across receivers, so that traversals run with full warps. VJP:
+// The last two occluders of pairs of this warp are tried first (ref_hit: a
+// triangle instead of a traversal), and what they do not block is queued,
+// across receivers, so that traversals run with full warps. VJP:
 // the sum of dL/dg * g / S^2, times 2 S, goes to the hit's material (per block
 // in shared memory first).
 // Bound by the pairs no kept occluder answers and by the pairs' own
-// arithmetic. 1e5 rays x 1000 receivers in the city: 1.73 ms, where a thread
-// per (ray, chunk of receivers) with a traversal per pair took 3.89 ms.
+// arithmetic. 1e5 rays x 1000 receivers in the city, mean of six sites: 1.37
+// ms, where a thread per (ray, chunk of receivers) with a traversal per pair
+// took 3.83 ms. (One occluder kept instead of two: 7 % slower; the queued
+// segments as beams: 4 % slower, they fan out over the receivers.)
 template <bool VJP, int LY>
 __global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
     extern __shared__ float sgrad[];
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
     const long long batches = (p.N + p.rays - 1) / p.rays;
     const long long units = (long long)p.n_tx * batches * p.n_chunks;
     TravCount cnt;
-    int ref = RT_NO_REF;   // an occluder of recent pairs
+    int ref0 = RT_NO_REF, ref1 = RT_NO_REF;   // the last two occluders of recent pairs
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
         const long long tb = u / p.n_chunks;
         const int chunk = (int)(u - tb * p.n_chunks);
@@ -255,8 +261,11 @@ __global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
                     const float4 hp = h.pt[k];
                     const f3 P = xyz(hp), v = rx - P;
                     const float dist = sqrtf(dot(v, v));
+                    const f3 ks = v * (1.0f / dist);
+                    const int hit = __float_as_int(hp.w);
                     if (dot(v, xyz(h.nm[k])) / dist > 0.0f)
-                        open = !ref_hit(p.s, ref, P, v * (1.0f / dist), dist - p.s.tmin, __float_as_int(hp.w), -1);
+                        open = !ref_hit(p.s, ref0, P, ks, dist - p.s.tmin, hit, -1) &&
+                               !ref_hit(p.s, ref1, P, ks, dist - p.s.tmin, hit, -1);
                 }
                 const unsigned om = __ballot_sync(full, open);
                 if (open) {
@@ -267,11 +276,11 @@ __global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
                 __syncwarp();
                 if (nq >= 32) {
                     nq -= 32;
-                    scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], nq, 32, t, sgrad, ref, cnt);
+                    scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], nq, 32, t, sgrad, ref0, ref1, cnt);
                 }
             }
         }
-        if (nq > 0) scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], 0, nq, t, sgrad, ref, cnt);
+        if (nq > 0) scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], 0, nq, t, sgrad, ref0, ref1, cnt);
     }
     if (VJP && p.grad_smem) {
         __syncthreads();
