@@ -901,14 +901,18 @@ float host_unord(unsigned u) {
 // `margin`.
 __global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tris, int n, int n_big, float margin,
                                                    int groups, int sets, float4* __restrict__ pk) {
-    float4 *b0 = pk + 2, *b1 = b0 + 64 * (size_t)groups, *b2 = b1 + 64 * (size_t)sets;
-    float4* bb = b2 + 64 * (size_t)((sets + 31) / 32);
+    const int b0 = 0, b1 = 32 * groups, b2 = b1 + 32 * sets, bb = b2 + (sets + 31) / 32 * 32;   // first records
+    const int records = bb + (n_big + 31) / 32 * 32;
     __shared__ float sb[32][6];
     const float inf = __int_as_float(0x7f800000);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto put = [](float4* p, const float (&b)[6], int ref) {
-        p[0] = make_float4(b[0], b[1], b[2], b[3]);
-        p[1] = make_float4(b[4], b[5], __int_as_float(ref), 0.0f);
+    auto put = [&](int rec, const float (&b)[6], int ref) {
+        for (int o = 0; o < 8; o++) {
+            float4* p = pk + 2 * (1 + (size_t)o * records + rec);
+            const int x = (o & 1) ? 3 : 0, y = (o & 2) ? 4 : 1, z = (o & 4) ? 5 : 2;   // entry planes
+            p[0] = make_float4(b[x], b[3 - x], b[y], b[5 - y]);
+            p[1] = make_float4(b[z], b[7 - z], __int_as_float(ref), 0.0f);
+        }
     };
     auto leaf = [&](int k, bool in, float (&b)[6]) {
         for (int q = 0; q < 3; q++) {
@@ -925,20 +929,20 @@ __global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tr
     };
     float b[6];
     if ((int)blockIdx.x == sets) {
-        if (threadIdx.x == 0) *reinterpret_cast<int4*>(pk) = make_int4(groups, sets, (n_big + 31) / 32 * 32, 0);
+        if (threadIdx.x == 0) *reinterpret_cast<int4*>(pk) = make_int4(groups, sets, (n_big + 31) / 32 * 32, records);
         for (int k = threadIdx.x; k < (n_big + 31) / 32 * 32; k += blockDim.x) {
             leaf(n + k, k < n_big, b);
-            put(bb + 2 * (size_t)k, b, n + k);
+            put(bb + k, b, n + k);
         }
         for (int k = sets + threadIdx.x; k < (sets + 31) / 32 * 32; k += blockDim.x) {
             leaf(0, false, b);
-            put(b2 + 2 * (size_t)k, b, 0);
+            put(b2 + k, b, 0);
         }
         return;
     }
     const int g = 32 * blockIdx.x + w, k = 32 * g + lane;
     leaf(k, k < n, b);
-    if (g < groups) put(b0 + 2 * (size_t)k, b, k);
+    if (g < groups) put(b0 + k, b, k);
     auto reduce = [&]() {
         for (int q = 0; q < 3; q++)
             for (int o = 16; o > 0; o >>= 1) {
@@ -948,14 +952,14 @@ __global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tr
     };
     reduce();
     if (lane == 0) {
-        put(b1 + 2 * (size_t)g, b, 0);
+        put(b1 + g, b, 0);
         for (int q = 0; q < 6; q++) sb[w][q] = b[q];
     }
     __syncthreads();
     if (w != 0) return;
     for (int q = 0; q < 6; q++) b[q] = sb[lane][q];
     reduce();
-    if (lane == 0) put(b2 + 2 * (size_t)blockIdx.x, b, 0);
+    if (lane == 0) put(b2 + blockIdx.x, b, 0);
 }
 
 int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
@@ -1217,7 +1221,7 @@ int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
     const int groups = (n + 31) / 32, sets = (groups + 31) / 32;
-    RT_TRY(buf_reserve(ctx->pk, 32 * (1 + 32 * ((size_t)groups + sets + (sets + 31) / 32 + (n_big + 31) / 32))));
+    RT_TRY(buf_reserve(ctx->pk, 32 * (1 + 8 * 32 * ((size_t)groups + sets + (sets + 31) / 32 + (n_big + 31) / 32))));
     prof_begin(ctx, "k_pk_boxes");
     k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), n, (int)n_big, 4e-6f * ext, groups, sets,
                                           bp<float4>(ctx->pk));

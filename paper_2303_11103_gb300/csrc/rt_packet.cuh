@@ -14,10 +14,16 @@
 // boxes are widened (4e-6 of the scene's extent) beyond what rounding can
 // shift.
 //
-// Boxes at s.pk, 32-byte records: (groups, sets, large triangles rounded up to
-// 32); 32 leaves a group; 32 groups a set; the sets and the large triangles,
-// padded to multiples of 32 by boxes no beam meets. A record holds lo, hi and,
-// for a triangle, its index in s.tris.
+// Boxes at s.pk, 32-byte records: first (groups, sets, large triangles rounded
+// up to 32, records of a copy), then 8 copies, one for each octant of
+// directions, of: 32 leaves a group; 32 groups a set; the sets and the large
+// triangles, padded to multiples of 32 by boxes no beam meets. A record holds
+// the entry and exit planes of its octant in pairs (lo and hi where the
+// direction is positive, hi and lo where it is negative) and, for a triangle,
+// its index in s.tris. With the planes in this order a box test is three packed
+// FMAs and four min / max; with one copy of lo and hi, chosen between and
+// subtracted in the test, it took three times the instructions (64-transmitter
+// map 99.4 ms, 92.7 with the copies).
 #pragma once
 #include "rt_common.cuh"
 
@@ -50,7 +56,7 @@ __device__ __forceinline__ float warp_max(float x) {
 // as for a ray; where they part, both bound the entry (open), and where they
 // close in, both the exit (shut).
 struct BeamAxis {
-    float on, rn, of, rf;   // origin and reciprocal slope for the two planes
+    float2 r, c;            // reciprocal slopes and -origin * slope, for the entry and the exit plane
     bool neg, open, shut;   // neg: the entry plane is hi
 };
 struct Beam {
@@ -65,10 +71,8 @@ __device__ __forceinline__ BeamAxis beam_axis(float olo, float ohi, float dlo, f
     a.open = dlo < 0.0f && dhi > 0.0f;
     a.shut = dlo > 0.0f && dhi < 0.0f;
     const float rhi = __fdividef(1.0f, dhi > 0.0f || (dlo >= 0.0f && !a.shut) ? fmaxf(dhi, 1e-30f) : fminf(dhi, -1e-30f));
-    a.on = a.neg ? olo : ohi;
-    a.rn = a.neg ? rlo : rhi;
-    a.of = a.neg ? ohi : olo;
-    a.rf = a.neg ? rhi : rlo;
+    a.r = a.neg ? make_float2(rlo, rhi) : make_float2(rhi, rlo);
+    a.c = a.neg ? make_float2(-olo * rlo, -ohi * rhi) : make_float2(-ohi * rhi, -olo * rlo);
     return a;
 }
 // rays: origin and direction
@@ -85,16 +89,15 @@ __device__ __forceinline__ BeamAxis seg_axis(bool mine, float o, float e) {
     return beam_axis(olo, ohi, warp_min(mine ? e : inf) - olo, warp_max(mine ? e : -inf) - ohi);
 }
 
-// Where the beam enters box k of a level (bits of the distance, or of +inf
-// when it misses the box before tmax). ref: the record's triangle.
-__device__ __forceinline__ unsigned beam_box(const Beam& b, const float4* box, int k, float tmin, float tmax, int& ref) {
+// Where the beam enters a record's box (bits of the distance, or of +inf when
+// it misses the box before tmax). ref: the record's triangle.
+__device__ __forceinline__ unsigned beam_box(const Beam& b, const float4* box, float tmin, float tmax, int& ref) {
     const float inf = __int_as_float(0x7f800000);
     float4 p, q;
-    ldg8(box + 2 * (size_t)k, p, q);
+    ldg8(box, p, q);
     ref = __float_as_int(q.z);
-    const float nx = ((b.x.neg ? p.w : p.x) - b.x.on) * b.x.rn, fx = ((b.x.neg ? p.x : p.w) - b.x.of) * b.x.rf;
-    const float ny = ((b.y.neg ? q.x : p.y) - b.y.on) * b.y.rn, fy = ((b.y.neg ? p.y : q.x) - b.y.of) * b.y.rf;
-    const float nz = ((b.z.neg ? q.y : p.z) - b.z.on) * b.z.rn, fz = ((b.z.neg ? p.z : q.y) - b.z.of) * b.z.rf;
+    const float2 x = fma2(p.x, p.y, b.x.r, b.x.c), y = fma2(p.z, p.w, b.y.r, b.y.c), z = fma2(q.x, q.y, b.z.r, b.z.c);
+    const float nx = x.x, fx = x.y, ny = y.x, fy = y.y, nz = z.x, fz = z.y;
     float tn = fmax3(nx, ny, fmaxf(nz, tmin)), tf;
     if (!b.odd) {
         tf = fmin3(fx, fy, fminf(fz, tmax));
@@ -135,7 +138,9 @@ __device__ __forceinline__ void beam_walk(const DevScene& s, const Beam& b, bool
         return __reduce_max_sync(full, mine && !(any && id >= 0) ? __float_as_uint(SEG ? 1.0f : t) : 0u);
     };
     unsigned far = far_of();
-    const int4 n = __ldg(reinterpret_cast<const int4*>(s.pk));   // groups, sets, large triangles
+    const int4 n = __ldg(reinterpret_cast<const int4*>(s.pk));   // groups, sets, large triangles, records
+    const int oct = (b.x.neg ? 1 : 0) | (b.y.neg ? 2 : 0) | (b.z.neg ? 4 : 0);
+    const float4* boxes = s.pk + 2 * (1 + (size_t)oct * n.w + lane);
     const int r1 = 32 * n.x, r2 = r1 + 32 * n.y, rb = r2 + (n.y + 31) / 32 * 32;   // first records of the levels
     unsigned key1 = 0x7f800000u, key2 = 0x7f800000u;
     int level = 2, rec = r2, next2 = r2, next1 = 0;   // the round's level and first record; those of key2, key1
@@ -154,7 +159,7 @@ __device__ __forceinline__ void beam_walk(const DevScene& s, const Beam& b, bool
             }
         }
         int ref;
-        unsigned key = beam_box(b, s.pk + 2, rec + lane, SEG ? 0.0f : tmin, __uint_as_float(far), ref);
+        unsigned key = beam_box(b, boxes + 2 * (size_t)rec, SEG ? 0.0f : tmin, __uint_as_float(far), ref);
         if (level == 2) {
             key2 = key;
         } else if (level == 1) {
