@@ -65,7 +65,8 @@ struct DiffFind {
     const float* rx_pos;
     const int32_t* rx_off;   // [n_tx+1] or null
     int n_tx, n_rx;
-    int tiles, runs;         // receiver tiles of 32 (of the largest receiver set), runs of DF_RUN tiles
+    int tiles, runs;         // receiver tiles of 32 (of the largest receiver set), runs of run_len tiles
+    int run_len, take;       // units a warp takes at a time
     CellGrid grid;           // receivers at cell centres when grid.nx > 0
     unsigned long long* count;
     unsigned long long* work;   // units taken (cleared with the count)
@@ -129,12 +130,11 @@ __device__ __forceinline__ void diff_tail(const DiffFind& p, const int* qr, cons
     __syncwarp();
 }
 
-// Receiver tiles of a work unit, and cells of a grid tile (8 x 4: neighbouring
+// Receiver tiles of a work unit at most, and cells of a grid tile (8 x 4: neighbouring
 // cells see a wedge past the same occluders).
 constexpr int DF_RUN = 64;
 constexpr int DF_TX = 8, DF_TY = 4;
 constexpr int DF_Q = 64;   // entries of a warp's queues
-constexpr int DF_UNITS = 4;   // units a warp takes at a time
 
 // Whether some cell of a grid tile may have its Keller point on the edge
 // (0 < t < len): t = ts + (tr - ts) rs / (rs + rr) for the extremes of tr
@@ -169,7 +169,7 @@ __device__ __forceinline__ bool tile_reached(const CellGrid& g, int tile, int ti
 // The queued segments of a warp lie side by side (one wedge, neighbouring cells)
 // and go through the scene as a beam (warp_segments). Tiles of a map whose cells
 // all have their Keller point off the edge are left out, 32 of them tested at a
-// time. Units are handed out DF_UNITS at a time: dealt in turn they left some
+// time. Units are handed out as warps ask: dealt in turn they left some
 // SMs with twice the others' work.
 //
 // Bound by the candidates' own arithmetic and by the segments no kept
@@ -192,10 +192,10 @@ __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
     while (true) {
         if (u == u_end) {
             unsigned long long b = 0;
-            if (lane == 0) b = atomicAdd(p.work, (unsigned long long)DF_UNITS);
+            if (lane == 0) b = atomicAdd(p.work, (unsigned long long)p.take);
             u = (int64_t)__shfl_sync(full, b, 0);
             if (u >= units) break;
-            u_end = min(u + DF_UNITS, units);
+            u_end = min(u + p.take, units);
         }
         const int64_t tr_ = u / p.n_w;
         const int wi = (int)(u - tr_ * p.n_w);
@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(128) k_diff_find(DiffFind p) {
         const int f0 = __float_as_int(w.t0.w), f1 = __float_as_int(w.n0.w);
         int ref1 = RT_NO_REF, ref2 = RT_NO_REF;   // last occluders of tx -> D and D -> rx
         int n1 = 0, n2 = 0;                       // queued candidates (warp-uniform)
-        const int tile_end = min(p.tiles, (run + 1) * DF_RUN);
-        int next = run * DF_RUN;       // tiles not yet looked at, 32 at a time
+        const int tile_end = min(p.tiles, (run + 1) * p.run_len);
+        int next = run * p.run_len;       // tiles not yet looked at, 32 at a time
         int base = next;
         unsigned todo = 0;             // tiles base + k that may have a path
         while (true) {
@@ -525,10 +525,16 @@ __global__ void __launch_bounds__(64) k_diff_field(DiffField c, float2* __restri
 }  // namespace
 
 static void launch_diff_find(rt_ctx* ctx, DiffFind& p) {
-    p.runs = (p.tiles + DF_RUN - 1) / DF_RUN;
-    const int64_t units = (int64_t)p.n_tx * p.runs * p.n_w;
     const auto kern = wide_layout(ctx) ? k_diff_find<8> : k_diff_find<2>;
     const int64_t fit = (int64_t)std::max(1, blocks_per_sm((const void*)kern, 128, 0)) * ctx->num_sms;
+    // runs as long as leave every warp 8 units (a wedge's record, its kept
+    // occluders and the queues' last turns are per run; a map of 108 x 29 cells
+    // over 2700 wedges in runs of 64 kept half of the warps without work)
+    p.run_len = DF_RUN;
+    while (p.run_len > 2 && (int64_t)p.n_tx * p.n_w * ((p.tiles + p.run_len - 1) / p.run_len) < 8 * 4 * fit) p.run_len /= 2;
+    p.runs = (p.tiles + p.run_len - 1) / p.run_len;
+    const int64_t units = (int64_t)p.n_tx * p.runs * p.n_w;
+    p.take = units >= 64 * 4 * fit ? 4 : 1;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((units + 3) / 4, fit));
     prof_begin(ctx, "k_diff_find");
     kern<<<(unsigned)blocks, 128, 0, ctx->stream>>>(p);
