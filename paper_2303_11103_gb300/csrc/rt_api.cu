@@ -480,6 +480,30 @@ int rt_compute_paths(rt_ctx* ctx, int32_t max_depth, int64_t num_rays, uint32_t 
     return compute_paths_impl(ctx, max_depth, num_rays, flags, num_paths);
 }
 
+}  // extern "C"
+
+namespace {
+// Up to five arrays of 4-byte words copied in one launch (a copy each took
+// 1.5 us of device time and its own launch).
+struct CopySet {
+    const uint32_t* src[5];
+    uint32_t* dst[5];
+    int64_t end[5];   // words of this array and those before it
+    int n;
+};
+__global__ void k_copy_set(CopySet c) {
+    const int64_t total = c.n ? c.end[c.n - 1] : 0, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
+        int k = 0;
+        while (i >= c.end[k]) k++;
+        const int64_t j = i - (k ? c.end[k - 1] : 0);
+        c.dst[k][j] = c.src[k][j];
+    }
+}
+}  // namespace
+
+extern "C" {
+
 int rt_get_paths(rt_ctx* ctx, int64_t* offsets, int32_t* seq, float* points, int32_t* depth, double* length) {
     CHECK_CTX(ctx);
     int64_t np = 0;
@@ -487,13 +511,30 @@ int rt_get_paths(rt_ctx* ctx, int64_t* offsets, int32_t* seq, float* points, int
     const int64_t P = ctx->n_paths;
     const int D = ctx->max_depth;
     cudaStream_t st = ctx->stream;
-    if (offsets) RT_TRY(cudaMemcpyAsync(offsets, ctx->path_off.p, sizeof(int64_t) * (np + 1), cudaMemcpyDeviceToDevice, st));
-    if (P > 0) {
-        if (seq) RT_TRY(cudaMemcpyAsync(seq, ctx->path_seq.p, sizeof(int32_t) * P * D, cudaMemcpyDeviceToDevice, st));
-        if (points) RT_TRY(cudaMemcpyAsync(points, ctx->path_pts.p, sizeof(float) * 3 * P * D, cudaMemcpyDeviceToDevice, st));
-        if (depth) RT_TRY(cudaMemcpyAsync(depth, ctx->path_depth.p, sizeof(int32_t) * P, cudaMemcpyDeviceToDevice, st));
-        if (length) RT_TRY(cudaMemcpyAsync(length, ctx->path_len.p, sizeof(double) * P, cudaMemcpyDeviceToDevice, st));
+    CopySet c;
+    c.n = 0;
+    const struct { void* dst; const DevBuf* src; size_t bytes; } arrays[5] = {
+        {offsets, &ctx->path_off, sizeof(int64_t) * (size_t)(np + 1)},
+        {seq, &ctx->path_seq, sizeof(int32_t) * (size_t)(P * D)},
+        {points, &ctx->path_pts, sizeof(float) * 3 * (size_t)(P * D)},
+        {depth, &ctx->path_depth, sizeof(int32_t) * (size_t)P},
+        {length, &ctx->path_len, sizeof(double) * (size_t)P}};
+    for (const auto& a : arrays) {
+        if (!a.dst || a.bytes == 0) continue;
+        if (a.bytes > a.src->bytes || (uintptr_t)a.dst % 4) {   // not computed for these devices, or not on a word boundary
+            RT_TRY(cudaMemcpyAsync(a.dst, a.src->p, a.bytes, cudaMemcpyDeviceToDevice, st));
+            continue;
+        }
+        c.src[c.n] = static_cast<const uint32_t*>(a.src->p);
+        c.dst[c.n] = static_cast<uint32_t*>(a.dst);
+        c.end[c.n] = (int64_t)(a.bytes / 4) + (c.n ? c.end[c.n - 1] : 0);
+        c.n++;
     }
+    if (c.n == 0) return RT_OK;
+    prof_begin(ctx, "k_copy_set");
+    k_copy_set<<<(unsigned)std::min<int64_t>((c.end[c.n - 1] + 255) / 256, 8 * ctx->num_sms), 256, 0, st>>>(c);
+    prof_end(ctx);
+    RT_TRY(cudaGetLastError());
     return RT_OK;
 }
 

@@ -178,9 +178,10 @@ inline size_t staged_bytes(const rt_ctx* c) {
 }
 
 // radix sort of 64-bit keys with an optional 32-bit payload, bits [0, end_bit)
-// result in keys/vals (alt buffers used as ping-pong), n may be 0
+// result in keys/vals, or with into_alt in the alt buffers (the other ones are
+// scratch), n may be 0
 cudaError_t radix_sort64(rt_ctx* ctx, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals,
-                         uint32_t* vals_alt, int64_t n, int end_bit);
+                         uint32_t* vals_alt, int64_t n, int end_bit, bool into_alt = false);
 
 cudaError_t exclusive_scan_u32(rt_ctx* ctx, uint32_t* a, int64_t m);
 

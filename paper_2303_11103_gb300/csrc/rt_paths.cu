@@ -90,12 +90,37 @@ struct KeyFmt {
     }
 };
 
-// LOS keys after the shooting keys: at `at`, or at *at_dev when given (the
-// shooting pass's key count, still on the device)
-__global__ void k_write_los(uint64_t* keys, uint32_t* vals, int64_t at, const unsigned long long* at_dev, int n_tx,
-                            KeyFmt f) {
+// What a call counts into, and the hash table's slots, cleared in one launch
+// (seven memsets of 2 to 3 us each before): counters and status null: the table
+// alone.
+__global__ void k_paths_clear(unsigned long long* counters, unsigned* status, uint4* __restrict__ tab,
+                              uint4* __restrict__ wit, int64_t S, uint32_t* __restrict__ cnt) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (i0 == 0) {
+        if (counters) counters[RT_CNT_WORK] = counters[RT_CNT_PATHS] = counters[RT_CNT_KEYS] = 0;
+        if (status) *status = 0;
+    }
+    if (S == 0) return;
+    if (i0 < 4) cnt[i0] = 0;
+    const uint4 ones = make_uint4(~0u, ~0u, ~0u, ~0u);
+    for (int64_t i = i0; i < S / 2; i += step) tab[i] = ones;
+    for (int64_t i = i0; i < S / 4; i += step) wit[i] = ones;
+}
+
+// Counts of a call to pinned host memory: keys shot, paths, distinct keys and
+// the hash table's overflow flag, status. One launch instead of a copy each.
+__global__ void k_paths_report(const unsigned long long* counters, const uint32_t* U, const uint32_t* overflow,
+                               const unsigned* status, uint64_t* host) {
+    host[0] = counters[RT_CNT_KEYS];
+    host[1] = counters[RT_CNT_PATHS];
+    host[2] = *U;
+    host[3] = overflow ? *overflow : 0;
+    host[4] = *status;
+}
+
+// LOS keys after the n shooting keys (the hash pass makes them itself)
+__global__ void k_write_los(uint64_t* keys, uint32_t* vals, int64_t at, int n_tx, KeyFmt f) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (at_dev) at = (int64_t)*at_dev;
     if (t < n_tx) {
         keys[at + t] = (uint64_t)t << f.tx_shift;
         vals[at + t] = 0xFFFFFFFFu;
@@ -119,19 +144,6 @@ __global__ void k_dedup_minwit(const uint64_t* __restrict__ k, const uint32_t* _
     }
 }
 
-// per-tx candidate ranges: off[t] = first candidate with tx >= t
-__global__ void k_cand_off(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ Up, int n_tx, KeyFmt f,
-                           int64_t* __restrict__ off) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t > n_tx) return;
-    int64_t lo = 0, hi = *Up;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (f.tx(ck[mid]) < t) lo = mid + 1; else hi = mid;
-    }
-    off[t] = lo;
-}
-
 // ---------------------------------------------------- hash duplicate removal
 // Candidate keys into an open-addressing table (linear probing, size a
 // power of two at least twice the key count, empty slots all ones, which no
@@ -148,28 +160,30 @@ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
     return x;
 }
 
-// n_dev (optional): the key count is *n_dev + n on the device; when it
-// exceeds cap (a table sized from an earlier call), nothing is inserted and
+// The n shooting keys are followed by one LOS key of each of n_los
+// transmitters. n_dev (optional): n is *n_dev, on the device; when all keys
+// exceed cap (a table sized from an earlier call), nothing is inserted and
 // *overflow is set, so that the host repeats the pass with the count read.
 __global__ void k_hash_insert(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals, int64_t n,
-                              const unsigned long long* __restrict__ n_dev, int64_t cap, unsigned* __restrict__ overflow,
-                              unsigned long long* __restrict__ tab, unsigned* __restrict__ wit, uint64_t mask) {
+                              const unsigned long long* __restrict__ n_dev, int n_los, int tx_shift, int64_t cap,
+                              unsigned* __restrict__ overflow, unsigned long long* __restrict__ tab,
+                              unsigned* __restrict__ wit, uint64_t mask) {
     // rays of one warp are coherent, so equal keys are merged in the warp first
     // (one table access and one atomicMin per distinct key of the warp)
     if (n_dev) {
-        n += (int64_t)*n_dev;
-        if (n > cap) {
+        n = (int64_t)*n_dev;
+        if (n + n_los > cap) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(overflow, 1u);
             return;
         }
     }
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n + n_los; base += stride) {
         const int64_t i = base + lane;
-        const bool ok = i < n;
-        const unsigned long long k = ok ? keys[i] : ~0ull;
-        const unsigned v = ok ? vals[i] : 0xFFFFFFFFu;
+        const bool ok = i < n + n_los;
+        const unsigned long long k = i < n ? keys[i] : ok ? (unsigned long long)(i - n) << tx_shift : ~0ull;
+        const unsigned v = i < n ? vals[i] : 0xFFFFFFFFu;
         const unsigned grp = __match_any_sync(0xffffffffu, k);
         const unsigned vmin = __reduce_min_sync(grp, v);
         if (!ok || lane != __ffs(grp) - 1) continue;
@@ -221,22 +235,23 @@ __device__ __forceinline__ void cand_img_one(const uint64_t* __restrict__ ck, in
     }
 }
 
-
-__global__ void k_cand_img(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ Up, KeyFmt f,
-                           const float* __restrict__ tx_pos, const float4* __restrict__ planes,
-                           float* __restrict__ img) {
-    const int64_t U = *Up;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < U; c += (int64_t)gridDim.x * blockDim.x)
-        cand_img_one(ck, c, f, tx_pos, planes, img);
-}
-
-// Validation work offsets in warp units: work_off[t] = sum over t' < t of
-// U_t' ceil(R_t' / 32), a unit being one candidate against 32 receivers (one
-// block; n_tx entries scanned in thread-contiguous runs).
-__global__ void __launch_bounds__(1024) k_work_off(const int64_t* __restrict__ cand_off,
-                                                   const int32_t* __restrict__ rx_off, int n_tx, int n_rx,
-                                                   int64_t* __restrict__ work_off) {
+// By one block: per-tx candidate ranges, cand_off[t] = first candidate with
+// tx >= t, then the validation work offsets in warp units, work_off[t] = sum
+// over t' < t of U_t' ceil(R_t' / 32), a unit being one candidate against 32
+// receivers (n_tx entries scanned in thread-contiguous runs).
+__device__ __forceinline__ void cand_ranges(const uint64_t* __restrict__ ck, int64_t U, KeyFmt f,
+                                            const int32_t* __restrict__ rx_off, int n_tx, int n_rx, int64_t* cand_off,
+                                            int64_t* work_off) {
     __shared__ long long ws[32];
+    for (int t = threadIdx.x; t <= n_tx; t += blockDim.x) {
+        int64_t lo = 0, hi = U;
+        while (lo < hi) {
+            int64_t mid = (lo + hi) >> 1;
+            if (f.tx(ck[mid]) < t) lo = mid + 1; else hi = mid;
+        }
+        cand_off[t] = lo;
+    }
+    __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int seg = (n_tx + (int)blockDim.x - 1) / (int)blockDim.x;
     const int s0 = min((int)threadIdx.x * seg, n_tx), s1 = min(s0 + seg, n_tx);
@@ -268,6 +283,19 @@ __global__ void __launch_bounds__(1024) k_work_off(const int64_t* __restrict__ c
         run += (cand_off[t + 1] - cand_off[t]) * R;
     }
     if (threadIdx.x == blockDim.x - 1) work_off[n_tx] = run;
+}
+
+// What the validation reads of the sorted candidates: block 0 the ranges, all
+// blocks the images.
+__global__ void __launch_bounds__(256) k_cand_prep(const uint64_t* __restrict__ ck, const uint32_t* __restrict__ Up,
+                                                   KeyFmt f, const float* __restrict__ tx_pos,
+                                                   const float4* __restrict__ planes, float* __restrict__ img,
+                                                   const int32_t* __restrict__ rx_off, int n_tx, int n_rx,
+                                                   int64_t* cand_off, int64_t* work_off) {
+    const int64_t U = *Up;
+    if (blockIdx.x == 0) cand_ranges(ck, U, f, rx_off, n_tx, n_rx, cand_off, work_off);
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < U; c += (int64_t)gridDim.x * blockDim.x)
+        cand_img_one(ck, c, f, tx_pos, planes, img);
 }
 
 // ------------------------------------------------------------ image method
@@ -517,11 +545,9 @@ __global__ void __launch_bounds__(256, 4) k_validate(ValParams p) {
     if (C) flush_counts(cnt, p.count - RT_CNT_PATHS, RT_CNT_ANY);
 }
 
-// offsets[p] = first path with pair >= p (paths sorted by pair, candidate)
-__global__ void k_path_off(const uint64_t* __restrict__ pk, int64_t P, int64_t n_pairs,
-                           int64_t* __restrict__ off) {
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q > n_pairs) return;
+// offsets[q] = first path with pair >= q (paths sorted by pair, candidate)
+__device__ __forceinline__ void path_off_one(const uint64_t* __restrict__ pk, int64_t P, int64_t q,
+                                             int64_t* __restrict__ off) {
     int64_t lo = 0, hi = P;
     uint64_t want = (uint64_t)q << 32;
     while (lo < hi) {
@@ -541,7 +567,8 @@ struct FinParams {
     const uint64_t* path_key;
     const int32_t* rx_off;
     int n_tx, n_rx;
-    int64_t P;
+    int64_t P, n_pairs;
+    int64_t* off;       // [n_pairs+1]
     int32_t* seq;
     float* pts;
     int32_t* depth;
@@ -549,11 +576,12 @@ struct FinParams {
     int32_t* pair_tx;   // [P*2]: tx, rx
 };
 
-// Reflection points (FP32) and path length accumulated in FP64: the length
+// Offsets of the pairs' paths, then reflection points (FP32) and path length accumulated in FP64: the length
 // of a specular path equals |rx - I_K| with I_K the last image of the
 // transmitter, computed here with FP64 planes from the FP32 vertices.
 __global__ void k_path_final(FinParams p) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i <= p.n_pairs) path_off_one(p.path_key, p.P, i, p.off);
     if (i >= p.P) return;
     uint64_t pk = p.path_key[i];
     int64_t pair = (int64_t)(pk >> 32);
@@ -632,9 +660,25 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
     RT_TRY(buf_reserve(ctx->vals_alt, sizeof(uint32_t) * std::max<int64_t>(ncap, 1)));
     uint64_t* keys = bp<uint64_t>(ctx->keys);
     uint32_t* vals = bp<uint32_t>(ctx->vals);
-    RT_TRY(cudaMemsetAsync(ctx->status.p, 0, sizeof(unsigned), st));
     int64_t nhit = 0;  // candidate keys the rays produced (one per hit)
-    bool fast = false;  // hash table sized from the previous call's key count
+    // the hash table sized from the previous call's key count, if there is one:
+    // the key count then stays on the device until the hash pass
+    bool fast = refl && ctx->dedup == RT_DEDUP_HASH && ctx->key_bits < 64 && ctx->hash_hint > 0;
+    RT_TRY(buf_reserve(ctx->htab_cnt, sizeof(uint32_t) * 4));
+    uint32_t* cntp = bp<uint32_t>(ctx->htab_cnt);   // [0] distinct keys, [1] overflow of a table sized beforehand
+    // clears the counters and the status (first), and a hash table of S slots
+    auto clear = [&](int64_t S, bool first) -> cudaError_t {
+        cudaError_t e = buf_reserve(ctx->htab_key, sizeof(uint64_t) * S);
+        if (e == cudaSuccess) e = buf_reserve(ctx->htab_wit, sizeof(uint32_t) * S);
+        if (e != cudaSuccess) return e;
+        prof_begin(ctx, "k_paths_clear");
+        k_paths_clear<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((S / 2 + 255) / 256, 8 * ctx->num_sms)), 256, 0, st>>>(
+            first ? bp<unsigned long long>(ctx->counters) : nullptr, first ? bp<unsigned>(ctx->status) : nullptr,
+            bp<uint4>(ctx->htab_key), bp<uint4>(ctx->htab_wit), S, cntp);
+        prof_end(ctx);
+        return cudaGetLastError();
+    };
+    RT_TRY(clear(fast ? ctx->hash_hint : 0, true));
     if (refl) {
         int32_t* hits = nullptr;
         if (ctx->recorded_rays) {
@@ -648,9 +692,6 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
         // that it shares the GPU with the refinement below, not with the trace
         e = side_launch(ctx);
         if (e) return e;
-        // the key count is read here only when no earlier call sized the
-        // hash table; otherwise it stays on the device until the hash pass
-        fast = ctx->dedup == RT_DEDUP_HASH && ctx->key_bits < 64 && ctx->hash_hint > 0;
         if (!fast) {
             RT_TRY(cudaMemcpyAsync(ctx->host_rb, bp<unsigned long long>(ctx->counters) + RT_CNT_KEYS,
                                    sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
@@ -661,14 +702,15 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
     const int64_t extra = los ? ctx->n_tx : 0;
     const unsigned long long* nhit_dev = bp<unsigned long long>(ctx->counters) + RT_CNT_KEYS;
     int64_t nkeys = nhit + extra;   // with fast: known after the hash pass
-    if (los) {
-        prof_begin(ctx, "k_write_los");
-        k_write_los<<<(ctx->n_tx + 255) / 256, 256, 0, st>>>(keys, vals, nhit, fast ? nhit_dev : nullptr, ctx->n_tx,
-                                                            f);
-        prof_end(ctx);
-        RT_TRY(cudaGetLastError());
-    }
     RT_TRY(buf_reserve(ctx->cand_off, sizeof(int64_t) * (ctx->n_tx + 1)));
+    auto report = [&](const uint32_t* U, const uint32_t* overflow) -> cudaError_t {
+        prof_begin(ctx, "k_paths_report");
+        k_paths_report<<<1, 1, 0, st>>>(bp<unsigned long long>(ctx->counters), U, overflow, bp<unsigned>(ctx->status),
+                                       ctx->host_rb);
+        prof_end(ctx);
+        const cudaError_t e = cudaGetLastError();
+        return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+    };
     const uint32_t* Ud = nullptr;   // device candidate count
     // hash table slots: a power of two, at least twice the keys
     auto slots_for = [](int64_t n) {
@@ -679,9 +721,6 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
     // beyond 2^29 slots (6 GB) the table would outgrow the sort's scratch: sort instead
     bool use_hash = ctx->key_bits < 64 && ctx->dedup == RT_DEDUP_HASH && (fast || slots_for(nkeys) <= (1ll << 29));
     if (use_hash) {
-        DevBuf& cnt = ctx->htab_cnt;
-        RT_TRY(buf_reserve(cnt, sizeof(uint32_t) * 4));
-        uint32_t* cntp = bp<uint32_t>(cnt);   // [0] distinct keys, [1] overflow of a table sized beforehand
         int64_t U = 0;
         for (int pass = 0; pass < 2; pass++) {
             const int64_t S = fast ? ctx->hash_hint : slots_for(nkeys);
@@ -690,35 +729,28 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             RT_TRY(buf_reserve(ctx->cand_wit, sizeof(uint32_t) * ucap));
             RT_TRY(buf_reserve(ctx->cand_img, sizeof(float) * 3 * f.D * ucap));
             // duplicate removal by hashing, then a sort of the distinct keys only
-            RT_TRY(buf_reserve(ctx->htab_key, sizeof(uint64_t) * S));
-            RT_TRY(buf_reserve(ctx->htab_wit, sizeof(uint32_t) * S));
-            RT_TRY(cudaMemsetAsync(ctx->htab_key.p, 0xFF, sizeof(uint64_t) * S, st));
-            RT_TRY(cudaMemsetAsync(ctx->htab_wit.p, 0xFF, sizeof(uint32_t) * S, st));
-            RT_TRY(cudaMemsetAsync(cnt.p, 0, sizeof(uint32_t) * 4, st));
+            if (!fast) RT_TRY(clear(S, false));
             if (fast || nkeys > 0) {
                 const int64_t span = fast ? S / 2 : nkeys;   // keys at most
                 prof_begin(ctx, "k_hash_insert");
                 k_hash_insert<<<(unsigned)std::min<int64_t>((span + 255) / 256, 8 * ctx->num_sms), 256, 0, st>>>(
-                    keys, vals, fast ? extra : nkeys, fast ? nhit_dev : nullptr, S / 2, cntp + 1,
+                    keys, vals, nhit, fast ? nhit_dev : nullptr, (int)extra, f.tx_shift, S / 2, cntp + 1,
                     bp<unsigned long long>(ctx->htab_key), bp<unsigned>(ctx->htab_wit), (uint64_t)(S - 1));
                 prof_end(ctx);
                 RT_TRY(cudaGetLastError());
                 prof_begin(ctx, "k_hash_compact");
                 k_hash_compact<<<(unsigned)((S + 255) / 256), 256, 0, st>>>(
                     bp<unsigned long long>(ctx->htab_key), bp<unsigned>(ctx->htab_wit), S,
-                    bp<uint64_t>(ctx->cand_key), bp<uint32_t>(ctx->cand_wit), cntp);
+                    bp<uint64_t>(ctx->keys_alt), bp<uint32_t>(ctx->vals_alt), cntp);
                 prof_end(ctx);
                 RT_TRY(cudaGetLastError());
             }
             // one read: distinct keys and overflow, and the shooting pass's key count
-            RT_TRY(cudaMemcpyAsync(ctx->host_rb, cntp, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-            if (fast)
-                RT_TRY(cudaMemcpyAsync(ctx->host_rb + 1, nhit_dev, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-            RT_TRY(cudaStreamSynchronize(st));
-            U = reinterpret_cast<uint32_t*>(ctx->host_rb)[0];
-            const bool overflow = reinterpret_cast<uint32_t*>(ctx->host_rb)[1] != 0;
+            RT_TRY(report(cntp, cntp + 1));
+            U = (int64_t)ctx->host_rb[2];
+            const bool overflow = ctx->host_rb[3] != 0;
             if (fast) {
-                nhit = (int64_t)ctx->host_rb[1];
+                nhit = (int64_t)ctx->host_rb[0];
                 nkeys = nhit + extra;
                 fast = false;
                 if (overflow) {
@@ -732,13 +764,19 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
         }
         if (use_hash) {
             ctx->hash_hint = slots_for(nkeys);
-            RT_TRY(radix_sort64(ctx, bp<uint64_t>(ctx->cand_key), bp<uint64_t>(ctx->keys_alt),
-                                bp<uint32_t>(ctx->cand_wit), bp<uint32_t>(ctx->vals_alt), U, ctx->key_bits));
+            RT_TRY(radix_sort64(ctx, bp<uint64_t>(ctx->keys_alt), bp<uint64_t>(ctx->cand_key),
+                                bp<uint32_t>(ctx->vals_alt), bp<uint32_t>(ctx->cand_wit), U, ctx->key_bits, true));
             Ud = cntp;
         }
     }
     if (!use_hash) {
         ctx->hash_hint = 0;
+        if (los) {
+            prof_begin(ctx, "k_write_los");
+            k_write_los<<<(ctx->n_tx + 255) / 256, 256, 0, st>>>(keys, vals, nhit, ctx->n_tx, f);
+            prof_end(ctx);
+            RT_TRY(cudaGetLastError());
+        }
         const int64_t ucap = std::max<int64_t>(nkeys, 1);
         RT_TRY(buf_reserve(ctx->cand_key, sizeof(uint64_t) * ucap));
         RT_TRY(buf_reserve(ctx->cand_wit, sizeof(uint32_t) * ucap));
@@ -773,26 +811,16 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             RT_TRY(cudaGetLastError());
         }
     }
-    if (nkeys > 0) {
-        prof_begin(ctx, "k_cand_img");
-        k_cand_img<<<(unsigned)std::min<int64_t>((nkeys + 255) / 256, 8 * ctx->num_sms), 256, 0, st>>>(
-            bp<uint64_t>(ctx->cand_key), Ud, f, bp<float>(ctx->tx_pos), bp<float4>(ctx->planes),
-            bp<float>(ctx->cand_img));
-        prof_end(ctx);
-        RT_TRY(cudaGetLastError());
-    }
-    prof_begin(ctx, "k_cand_off");
-    k_cand_off<<<(ctx->n_tx + 256) / 256, 256, 0, st>>>(bp<uint64_t>(ctx->cand_key), Ud, ctx->n_tx, f,
-                                                         bp<int64_t>(ctx->cand_off));
-    prof_end(ctx);
-    RT_TRY(cudaGetLastError());
-    // validation work (sum over tx of U_t * R_t), offsets on the device
+    // candidate images, and the validation work (sum over tx of U_t * R_t) with
+    // its offsets on the device
     int64_t n_pairs = ctx->rx_sets ? (int64_t)ctx->rx_off[ctx->n_tx] : (int64_t)ctx->n_tx * ctx->n_rx;
     DevBuf& woffd = ctx->path_cap_dummy;
     RT_TRY(buf_reserve(woffd, sizeof(int64_t) * (ctx->n_tx + 1)));
-    prof_begin(ctx, "k_work_off");
-    k_work_off<<<1, 1024, 0, st>>>(bp<int64_t>(ctx->cand_off), ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr,
-                                   ctx->n_tx, ctx->n_rx, bp<int64_t>(woffd));
+    prof_begin(ctx, "k_cand_prep");
+    k_cand_prep<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((nkeys + 255) / 256, 8 * ctx->num_sms)), 256, 0, st>>>(
+        bp<uint64_t>(ctx->cand_key), Ud, f, bp<float>(ctx->tx_pos), bp<float4>(ctx->planes), bp<float>(ctx->cand_img),
+        ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr, ctx->n_tx, ctx->n_rx, bp<int64_t>(ctx->cand_off),
+        bp<int64_t>(woffd));
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
     if (ctx->path_cap == 0) ctx->path_cap = 1 << 16;
@@ -800,7 +828,8 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
     for (int attempt = 0; attempt < 2; attempt++) {
         RT_TRY(buf_reserve(ctx->path_key, sizeof(uint64_t) * ctx->path_cap));
         RT_TRY(buf_reserve(ctx->path_key_alt, sizeof(uint64_t) * ctx->path_cap));
-        RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long) * 2, st));
+        if (attempt > 0)
+            RT_TRY(cudaMemsetAsync(bp<unsigned long long>(ctx->counters) + RT_CNT_PATHS, 0, sizeof(unsigned long long), st));
         if (nkeys > 0 && n_pairs > 0) {
             ValParams vp;
             vp.s = dev_scene(ctx);
@@ -814,7 +843,7 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             vp.rx_off = ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr;
             vp.n_tx = ctx->n_tx;
             vp.n_rx = ctx->n_rx;
-            vp.out = bp<uint64_t>(ctx->path_key);
+            vp.out = bp<uint64_t>(ctx->path_key_alt);
             vp.count = bp<unsigned long long>(ctx->counters) + 1;
             vp.cap = ctx->path_cap;
             vp.n_sm = staged_nodes(ctx);
@@ -834,16 +863,10 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             RT_TRY(cudaGetLastError());
         }
         // one read: path count, candidate count, status
-        RT_TRY(cudaMemcpyAsync(ctx->host_rb, bp<unsigned long long>(ctx->counters) + 1, sizeof(uint64_t),
-                               cudaMemcpyDeviceToHost, st));
-        RT_TRY(cudaMemcpyAsync(reinterpret_cast<uint32_t*>(ctx->host_rb + 1), Ud, sizeof(uint32_t),
-                               cudaMemcpyDeviceToHost, st));
-        RT_TRY(cudaMemcpyAsync(reinterpret_cast<uint32_t*>(ctx->host_rb + 2), ctx->status.p, sizeof(uint32_t),
-                               cudaMemcpyDeviceToHost, st));
-        RT_TRY(cudaStreamSynchronize(st));
-        P = (int64_t)ctx->host_rb[0];
-        ctx->n_cand = *reinterpret_cast<uint32_t*>(ctx->host_rb + 1);
-        const unsigned hs = *reinterpret_cast<uint32_t*>(ctx->host_rb + 2);
+        RT_TRY(report(Ud, nullptr));
+        P = (int64_t)ctx->host_rb[1];
+        ctx->n_cand = (int64_t)ctx->host_rb[2];
+        const unsigned hs = (unsigned)ctx->host_rb[4];
         if (hs & RT_STAT_STACK) return set_err(ctx, RT_ERR_CAPACITY, "traversal stack overflow");
         if (hs & RT_STAT_LOOP) return set_err(ctx, RT_ERR_CUDA, "malformed BVH (traversal budget exceeded)");
         if (hs & RT_STAT_SORT) return set_err(ctx, RT_ERR_TIMEOUT, "radix sort: tile look-back timed out");
@@ -853,43 +876,38 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
     ctx->n_paths = P;
     int pair_bits = 1;
     while ((1ll << pair_bits) < std::max<int64_t>(n_pairs, 2)) pair_bits++;
-    RT_TRY(radix_sort64(ctx, bp<uint64_t>(ctx->path_key), bp<uint64_t>(ctx->path_key_alt), nullptr, nullptr, P,
-                        32 + pair_bits));
+    RT_TRY(radix_sort64(ctx, bp<uint64_t>(ctx->path_key_alt), bp<uint64_t>(ctx->path_key), nullptr, nullptr, P,
+                        32 + pair_bits, true));
     RT_TRY(buf_reserve(ctx->path_off, sizeof(int64_t) * (n_pairs + 1)));
-    prof_begin(ctx, "k_path_off");
-    k_path_off<<<(unsigned)((n_pairs + 256) / 256), 256, 0, st>>>(bp<uint64_t>(ctx->path_key), P, n_pairs,
-                                                                  bp<int64_t>(ctx->path_off));
-    prof_end(ctx);
-    RT_TRY(cudaGetLastError());
     int64_t Pm = std::max<int64_t>(P, 1);
     RT_TRY(buf_reserve(ctx->path_seq, sizeof(int32_t) * Pm * f.D));
     RT_TRY(buf_reserve(ctx->path_pts, sizeof(float) * 3 * Pm * f.D));
     RT_TRY(buf_reserve(ctx->path_depth, sizeof(int32_t) * Pm));
     RT_TRY(buf_reserve(ctx->path_len, sizeof(double) * Pm));
     RT_TRY(buf_reserve(ctx->path_pair, sizeof(int32_t) * 2 * Pm));
-    if (P > 0) {
-        FinParams fp;
-        fp.s = dev_scene(ctx);
-        fp.f = f;
-        fp.tx_pos = bp<float>(ctx->tx_pos);
-        fp.rx_pos = bp<float>(ctx->rx_pos);
-        fp.cand_key = bp<uint64_t>(ctx->cand_key);
-        fp.cand_img = bp<float>(ctx->cand_img);
-        fp.path_key = bp<uint64_t>(ctx->path_key);
-        fp.rx_off = ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr;
-        fp.n_tx = ctx->n_tx;
-        fp.n_rx = ctx->n_rx;
-        fp.P = P;
-        fp.seq = bp<int32_t>(ctx->path_seq);
-        fp.pts = bp<float>(ctx->path_pts);
-        fp.depth = bp<int32_t>(ctx->path_depth);
-        fp.len = bp<double>(ctx->path_len);
-        fp.pair_tx = bp<int32_t>(ctx->path_pair);
-        prof_begin(ctx, "k_path_final");
-        k_path_final<<<(unsigned)((P + 127) / 128), 128, 0, st>>>(fp);
-        prof_end(ctx);
-        RT_TRY(cudaGetLastError());
-    }
+    FinParams fp;
+    fp.s = dev_scene(ctx);
+    fp.f = f;
+    fp.tx_pos = bp<float>(ctx->tx_pos);
+    fp.rx_pos = bp<float>(ctx->rx_pos);
+    fp.cand_key = bp<uint64_t>(ctx->cand_key);
+    fp.cand_img = bp<float>(ctx->cand_img);
+    fp.path_key = bp<uint64_t>(ctx->path_key);
+    fp.rx_off = ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr;
+    fp.n_tx = ctx->n_tx;
+    fp.n_rx = ctx->n_rx;
+    fp.P = P;
+    fp.n_pairs = n_pairs;
+    fp.off = bp<int64_t>(ctx->path_off);
+    fp.seq = bp<int32_t>(ctx->path_seq);
+    fp.pts = bp<float>(ctx->path_pts);
+    fp.depth = bp<int32_t>(ctx->path_depth);
+    fp.len = bp<double>(ctx->path_len);
+    fp.pair_tx = bp<int32_t>(ctx->path_pair);
+    prof_begin(ctx, "k_path_final");
+    k_path_final<<<(unsigned)((std::max(P, n_pairs + 1) + 127) / 128), 128, 0, st>>>(fp);
+    prof_end(ctx);
+    RT_TRY(cudaGetLastError());
     *out = P;
     return RT_OK;
 }

@@ -309,8 +309,8 @@ constexpr int RK_MAX = 256;   // up to this many keys: one-block rank sort
 // (stable); one shared-memory pass, no digit passes. Only the low end_bit
 // bits of the keys take part, as in the radix passes.
 template <bool VALS>
-__global__ void __launch_bounds__(RK_MAX) k_sort_rank(uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, int n,
-                                                     uint64_t mask) {
+__global__ void __launch_bounds__(RK_MAX) k_sort_rank(const uint64_t* keys, const uint32_t* vals, uint64_t* kout,
+                                                     uint32_t* vout, int n, uint64_t mask) {
     __shared__ uint64_t sk[RK_MAX];
     const int i = threadIdx.x;
     uint64_t k = 0;
@@ -329,10 +329,10 @@ __global__ void __launch_bounds__(RK_MAX) k_sort_rank(uint64_t* __restrict__ key
             r += (o < km) | ((o == km) & (j < i));
         }
     }
-    __syncthreads();   // every key has been read before the in-place writes
+    __syncthreads();   // every key has been read before the writes, which may be in place
     if (i < n) {
-        keys[r] = k;
-        if (VALS) vals[r] = v;
+        kout[r] = k;
+        if (VALS) vout[r] = v;
     }
 }
 
@@ -388,9 +388,20 @@ __global__ void __launch_bounds__(1024) k_sort_rank_multi(const uint64_t* __rest
 
 }  // namespace
 
+// The sorted keys where the caller wants them: copied from `k` unless they are there.
+static cudaError_t sort_result(rt_ctx* ctx, uint64_t* dst, const uint64_t* k, uint32_t* vdst, const uint32_t* v, int64_t n) {
+    if (dst == k || n == 0) return cudaSuccess;
+    cudaError_t e = cudaMemcpyAsync(dst, k, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
+    if (e == cudaSuccess && v)
+        e = cudaMemcpyAsync(vdst, v, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
+    return e;
+}
+
 cudaError_t radix_sort64(rt_ctx* ctx, uint64_t* keys, uint64_t* keys_alt, uint32_t* vals,
-                         uint32_t* vals_alt, int64_t n, int end_bit) {
-    if (n <= 1 || end_bit <= 0) return cudaSuccess;
+                         uint32_t* vals_alt, int64_t n, int end_bit, bool into_alt) {
+    uint64_t* kres = into_alt ? keys_alt : keys;
+    uint32_t* vres = into_alt ? vals_alt : vals;
+    if (n <= 1 || end_bit <= 0) return sort_result(ctx, kres, keys, vres, vals, n);
     if (n > (int64_t)0xFFFFFFFFll) return cudaErrorInvalidValue;
     if (n <= RK_MAX) {
         const int bits = 8 * ((end_bit + 7) / 8);   // the bits the digit passes would order by
@@ -398,9 +409,9 @@ cudaError_t radix_sort64(rt_ctx* ctx, uint64_t* keys, uint64_t* keys_alt, uint32
         const int threads = 32 * (int)((n + 31) / 32);
         prof_begin(ctx, "k_sort_rank");
         if (vals)
-            k_sort_rank<true><<<1, threads, 0, ctx->stream>>>(keys, vals, (int)n, mask);
+            k_sort_rank<true><<<1, threads, 0, ctx->stream>>>(keys, vals, kres, vres, (int)n, mask);
         else
-            k_sort_rank<false><<<1, threads, 0, ctx->stream>>>(keys, nullptr, (int)n, mask);
+            k_sort_rank<false><<<1, threads, 0, ctx->stream>>>(keys, nullptr, kres, nullptr, (int)n, mask);
         prof_end(ctx);
         return cudaGetLastError();
     }
@@ -426,10 +437,7 @@ cudaError_t radix_sort64(rt_ctx* ctx, uint64_t* keys, uint64_t* keys_alt, uint32
         prof_end(ctx);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(keys, keys_alt, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
-        if (e == cudaSuccess && vals)
-            e = cudaMemcpyAsync(vals, vals_alt, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
-        return e;
+        return sort_result(ctx, kres, keys_alt, vres, vals_alt, n);
     }
     int nb = (int)((n + RS_TILE - 1) / RS_TILE);
     const int passes_all = (end_bit + 7) / 8;
@@ -465,12 +473,7 @@ cudaError_t radix_sort64(rt_ctx* ctx, uint64_t* keys, uint64_t* keys_alt, uint32
             std::swap(kin, kout);
             std::swap(vin, vout);
         }
-        if (kin != keys) {
-            e = cudaMemcpyAsync(keys, kin, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
-            if (e != cudaSuccess) return e;
-            if (vals) e = cudaMemcpyAsync(vals, vin, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
-        }
-        return e;
+        return sort_result(ctx, kres, kin, vres, vin, n);
     }
     cudaError_t e = buf_reserve(ctx->sort_hist, sizeof(uint32_t) * 256 * (size_t)nb);
     if (e != cudaSuccess) return e;
@@ -496,12 +499,7 @@ cudaError_t radix_sort64(rt_ctx* ctx, uint64_t* keys, uint64_t* keys_alt, uint32
         uint64_t* tk = kin; kin = kout; kout = tk;
         uint32_t* tv = vin; vin = vout; vout = tv;
     }
-    if (kin != keys) {
-        e = cudaMemcpyAsync(keys, kin, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
-        if (e != cudaSuccess) return e;
-        if (vals) e = cudaMemcpyAsync(vals, vin, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream);
-    }
-    return e;
+    return sort_result(ctx, kres, kin, vres, vin, n);
 }
 
 // Exclusive scan of m uint32 entries in place.

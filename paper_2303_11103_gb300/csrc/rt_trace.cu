@@ -632,7 +632,8 @@ static bool use_beams(const rt_ctx* ctx, const TraceCommon& c) {
 }
 
 // Shoot and bounce: appends every hit's candidate key with its position
-// (tx*N + i)*D + depth; the key count goes to counter slot RT_CNT_KEYS.
+// (tx*N + i)*D + depth; the key count goes to counter slot RT_CNT_KEYS, which
+// the caller has cleared, with RT_CNT_WORK.
 int launch_sbr(rt_ctx* ctx, int64_t N, int D, uint64_t* keys, uint32_t* vals, int32_t* hits) {
     int e = ensure_perm(ctx, N);
     if (e) return e;
@@ -651,8 +652,6 @@ int launch_sbr(rt_ctx* ctx, int64_t N, int D, uint64_t* keys, uint32_t* vals, in
                                  : (ctx->count_work ? k_sbr<true, 2> : k_sbr<false, 2>);
     if (use_beams(ctx, p.c)) kern = k_sbr<false, 2, true>;
     RT_TRY(ensure_smem_attr((const void*)kern, smem));
-    RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), ctx->stream));
-    RT_TRY(cudaMemsetAsync(p.n_keys, 0, sizeof(unsigned long long), ctx->stream));
     int grid = trace_grid(ctx, (const void*)kern, smem);
     p.c.chunk = pick_chunk(ctx, p.c.total, grid);
     prof_begin(ctx, "k_sbr");
