@@ -73,22 +73,23 @@ __device__ float directive_norm(int alpha, float ci) {
     return ldexpf(tot, -alpha);
 }
 
-// Rays of a work unit at most, threads of a block, entries of a warp's queue.
-constexpr int SC_RAYS = 256, SC_THREADS = 128, SC_WARPS = SC_THREADS / 32, SC_Q = 64;
+// Rays of a work unit at most, entries of a warp's queue.
+constexpr int SC_RAYS = 256, SC_Q = 64;
 
-// A unit's scattering hits, in shared memory.
+// A unit's scattering hits (RAYS at most), in shared memory.
+template <int RAYS>
 struct ScatHits {
-    float4 pt[SC_RAYS];    // hit point, hit triangle
-    float4 nm[SC_RAYS];    // normal on the side the ray came from, material
-    float4 tx[SC_RAYS];    // transmit power of both ports, coefficient S, pattern exponent
-    float4 dir[SC_RAYS];   // specular direction, F_alpha / pi (directive patterns only)
+    float4 pt[RAYS];    // hit point, hit triangle
+    float4 nm[RAYS];    // normal on the side the ray came from, material
+    float4 tx[RAYS];    // transmit power of both ports, coefficient S, pattern exponent
+    float4 dir[RAYS];   // specular direction, F_alpha / pi (directive patterns only)
 };
 
 // Any occluder between a queued (hit, receiver) pair, then its contribution:
 // lane < take handles entry n + lane. Called by all 32 lanes; the occluder
 // found last goes to ref0, the one before it to ref1.
-template <bool VJP, int LY>
-__device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHits& h, const int* qr,
+template <bool VJP, int LY, int RAYS>
+__device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHits<RAYS>& h, const int* qr,
                                               const uint16_t* qh, int n, int take, int t, float* sgrad, int& ref0,
                                               int& ref1, TravCount& cnt) {
     const unsigned full = 0xffffffffu;
@@ -178,12 +179,16 @@ __device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHit
 // ms, where a thread per (ray, chunk of receivers) with a traversal per pair
 // took 3.83 ms. (One occluder kept instead of two: 7 % slower; the queued
 // segments as beams: 4 % slower, they fan out over the receivers.)
-template <bool VJP, int LY>
-__global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
+// W: warps of a block; 4, or 1 (with 32 rays a unit) where the receivers are few
+// and the first hits weigh as much as the pairs, so that no warp waits for
+// another's rays.
+template <bool VJP, int LY, int W>
+__global__ void __launch_bounds__(32 * W, W == 4 ? 7 : 28) k_scatter(ScatParams p) {
+    constexpr int RAYS = W == 1 ? 32 : SC_RAYS;
     extern __shared__ float sgrad[];
-    __shared__ ScatHits h;
-    __shared__ int q_rx[SC_WARPS][SC_Q];
-    __shared__ uint16_t q_hit[SC_WARPS][SC_Q];
+    __shared__ ScatHits<RAYS> h;
+    __shared__ int q_rx[W][SC_Q];
+    __shared__ uint16_t q_hit[W][SC_Q];
     __shared__ int n_hit;
     const unsigned full = 0xffffffffu, lt = lanemask_lt();
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
         __syncthreads();          // the last unit's hits are no longer read
         if (threadIdx.x == 0) n_hit = 0;
         __syncthreads();
-        for (int k0 = 0; k0 < p.rays; k0 += SC_THREADS) {
+        for (int k0 = 0; k0 < p.rays; k0 += 32 * W) {
             const long long i = i0 + k0 + threadIdx.x;
             const bool in = k0 + (int)threadIdx.x < p.rays && i < p.N;
             float sc = 0.0f, th = 0.0f;
@@ -252,35 +257,43 @@ __global__ void __launch_bounds__(SC_THREADS) k_scatter(ScatParams p) {
         __syncthreads();
         const int nh = n_hit;
         int nq = 0;   // queued pairs (warp-uniform)
-        for (int r = rb + wp; r < re; r += SC_WARPS) {
-            const f3 rx = mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
-            for (int k0 = 0; k0 < nh; k0 += 32) {
-                const int k = k0 + lane;
-                bool open = false;
-                if (k < nh) {
-                    const float4 hp = h.pt[k];
-                    const f3 P = xyz(hp), v = rx - P;
-                    const float dist = sqrtf(dot(v, v));
-                    const f3 ks = v * (1.0f / dist);
-                    const int hit = __float_as_int(hp.w);
-                    if (dot(v, xyz(h.nm[k])) / dist > 0.0f)
-                        open = !ref_hit(p.s, ref0, P, ks, dist - p.s.tmin, hit, -1) &&
-                               !ref_hit(p.s, ref1, P, ks, dist - p.s.tmin, hit, -1);
-                }
-                const unsigned om = __ballot_sync(full, open);
-                if (open) {
-                    q_rx[wp][nq + __popc(om & lt)] = r;
-                    q_hit[wp][nq + __popc(om & lt)] = (uint16_t)k;
-                }
-                nq += __popc(om);
-                __syncwarp();
-                if (nq >= 32) {
-                    nq -= 32;
-                    scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], nq, 32, t, sgrad, ref0, ref1, cnt);
-                }
+        // (receiver, 32 hits) in receiver order, an equal run of them for each warp
+        const int nt = (nh + 31) / 32;
+        const long long steps = (long long)(re - rb) * nt;
+        const long long step0 = steps * wp / W, step1 = steps * (wp + 1) / W;
+        int r = nt ? rb + (int)(step0 / nt) : rb, tile = nt ? (int)(step0 % nt) : 0;
+        f3 rx = mk(0, 0, 0);
+        for (long long step = step0; step < step1; step++) {
+            if (step == step0 || tile == 0) rx = mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
+            const int k = 32 * tile + lane;
+            bool open = false;
+            if (k < nh) {
+                const float4 hp = h.pt[k];
+                const f3 P = xyz(hp), v = rx - P;
+                const float dist = sqrtf(dot(v, v));
+                const f3 ks = v * (1.0f / dist);
+                const int hit = __float_as_int(hp.w);
+                if (dot(v, xyz(h.nm[k])) / dist > 0.0f)
+                    open = !ref_hit(p.s, ref0, P, ks, dist - p.s.tmin, hit, -1) &&
+                           !ref_hit(p.s, ref1, P, ks, dist - p.s.tmin, hit, -1);
+            }
+            const unsigned om = __ballot_sync(full, open);
+            if (open) {
+                q_rx[wp][nq + __popc(om & lt)] = r;
+                q_hit[wp][nq + __popc(om & lt)] = (uint16_t)k;
+            }
+            nq += __popc(om);
+            __syncwarp();
+            if (nq >= 32) {
+                nq -= 32;
+                scatter_batch<VJP, LY, RAYS>(p, h, q_rx[wp], q_hit[wp], nq, 32, t, sgrad, ref0, ref1, cnt);
+            }
+            if (++tile == nt) {
+                tile = 0;
+                r++;
             }
         }
-        if (nq > 0) scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], 0, nq, t, sgrad, ref0, ref1, cnt);
+        if (nq > 0) scatter_batch<VJP, LY, RAYS>(p, h, q_rx[wp], q_hit[wp], 0, nq, t, sgrad, ref0, ref1, cnt);
     }
     if (VJP && p.grad_smem) {
         __syncthreads();
@@ -327,29 +340,41 @@ int scattering_impl(rt_ctx* ctx, int64_t N, float* gain, const float* up, float*
     p.gain = gain;
     // work units: up to SC_RAYS rays against a chunk of the receivers. The rays
     // of a unit share its occluders and its chunk's receivers amortise their
-    // first hits, so both shrink only while the units would not fill the chip
-    // (2 x 1464 rays x 127 receivers: 0.17 ms; one thread per ray and 64
-    // receivers took 1.22 ms)
+    // first hits, so both shrink only while the units would not fill the chip:
+    // to 128 rays and 32 receivers for 16 units per SM, to 32 rays and 4 receivers
+    // for one wave (2 x 1464 rays x 127 receivers: 0.10 ms; one thread per ray and
+    // 64 receivers took 1.22 ms). Below 16 receivers a unit is a warp's 32 rays
+    // (1e5 rays x 1 receiver: 51 us, blocks of four warps 62)
     int nr_max = ctx->n_rx;
     if (ctx->rx_sets) {
         nr_max = 0;
         for (int t = 0; t < ctx->n_tx; t++) nr_max = std::max(nr_max, ctx->rx_off[t + 1] - ctx->rx_off[t]);
     }
-    const long long want = 16ll * ctx->num_sms;
+    const bool few = nr_max < 16;
+    const long long sms = ctx->num_sms, wave = (few ? 28 : 7) * sms;
     auto n_units = [&](int rays, long long chunks) { return (long long)ctx->n_tx * ((N + rays - 1) / rays) * chunks; };
-    const long long max_chunks = std::max(1, nr_max / 32);
-    p.rays = SC_RAYS;
-    while (p.rays > 32 && n_units(p.rays, max_chunks) < want) p.rays /= 2;
-    p.n_chunks = (int)std::max<long long>(1, std::min(max_chunks, (want + n_units(p.rays, 1) - 1) / n_units(p.rays, 1)));
-    const long long blocks = std::min<long long>(n_units(p.rays, p.n_chunks), 1ll << 30);
+    auto chunks_for = [&](int rays, long long units, int receivers) {
+        return std::max<long long>(1, std::min<long long>(nr_max / receivers, (units + n_units(rays, 1) - 1) / n_units(rays, 1)));
+    };
+    p.rays = few ? 32 : SC_RAYS;
+    if (!few && n_units(p.rays, std::max(1, nr_max / 32)) < 16 * sms) p.rays = 128;
+    p.n_chunks = (int)chunks_for(p.rays, 16 * sms, 32);
+    if (n_units(p.rays, p.n_chunks) < wave) p.n_chunks = (int)chunks_for(p.rays, wave, 4);
+    while (p.rays > 32 && n_units(p.rays, p.n_chunks) < wave) p.rays /= 2;
+    const unsigned blocks = (unsigned)std::min<long long>(n_units(p.rays, p.n_chunks), 1ll << 30);
+    const int threads = few ? 32 : 128;
+    const size_t smem = p.grad_smem ? sizeof(float) * ctx->n_mat : 0;
+    const bool wide = wide_layout(ctx);
     if (vjp) {
         prof_begin(ctx, "k_scatter_vjp");
-        auto kern = wide_layout(ctx) ? k_scatter<true, 8> : k_scatter<true, 2>;
-        kern<<<(unsigned)blocks, SC_THREADS, p.grad_smem ? sizeof(float) * ctx->n_mat : 0, ctx->stream>>>(p);
+        auto kern = few ? (wide ? k_scatter<true, 8, 1> : k_scatter<true, 2, 1>)
+                        : (wide ? k_scatter<true, 8, 4> : k_scatter<true, 2, 4>);
+        kern<<<blocks, threads, smem, ctx->stream>>>(p);
     } else {
         prof_begin(ctx, "k_scatter");
-        auto kern = wide_layout(ctx) ? k_scatter<false, 8> : k_scatter<false, 2>;
-        kern<<<(unsigned)blocks, SC_THREADS, 0, ctx->stream>>>(p);
+        auto kern = few ? (wide ? k_scatter<false, 8, 1> : k_scatter<false, 2, 1>)
+                        : (wide ? k_scatter<false, 8, 4> : k_scatter<false, 2, 4>);
+        kern<<<blocks, threads, 0, ctx->stream>>>(p);
     }
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
