@@ -344,16 +344,6 @@ __global__ void __launch_bounds__(256, 4) k_coverage(CovParams p) {
             tx = (int)t64;
             o = mk(p.c.tx_pos[3 * tx], p.c.tx_pos[3 * tx + 1], p.c.tx_pos[3 * tx + 2]);
             d = ray_dir(p.c, kd, i);
-            Rot<float> Rt;
-            if (rot_cached) {
-                for (int q = 0; q < 9; q++) Rt.m[q / 3][q % 3] = s_rot[9 * tx + q];
-            } else {
-                Rt = rot_ypr(p.c.tx_ypr[3 * tx], p.c.tx_ypr[3 * tx + 1], p.c.tx_ypr[3 * tx + 2]);
-            }
-            V3<float> f = antenna_vec<float>(p.txa.kind, zeta_t, Rt, V3<float>{d.x, d.y, d.z});
-            E[0] = {f.x, 0.0f};
-            E[1] = {f.y, 0.0f};
-            E[2] = {f.z, 0.0f};
             last = -1;
             depth = 0;
             alive = true;
@@ -367,6 +357,20 @@ __global__ void __launch_bounds__(256, 4) k_coverage(CovParams p) {
         const bool more = depth < p.D;
         const long long cell = cov_segment_warp<C, L, B>(p, sm, alive, tx, o, d, last, more, id, t, cnt, cnt_pl);
         if (alive) {
+            // the field at the transmitter, for rays that meet the map or a surface
+            // (about half of a mast's rays end in the sky)
+            if (depth == 0 && (cell >= 0 || (more && id >= 0))) {
+                Rot<float> Rt;
+                if (rot_cached) {
+                    for (int q = 0; q < 9; q++) Rt.m[q / 3][q % 3] = s_rot[9 * tx + q];
+                } else {
+                    Rt = rot_ypr(p.c.tx_ypr[3 * tx], p.c.tx_ypr[3 * tx + 1], p.c.tx_ypr[3 * tx + 2]);
+                }
+                V3<float> f = antenna_vec<float>(p.txa.kind, zeta_t, Rt, V3<float>{d.x, d.y, d.z});
+                E[0] = {f.x, 0.0f};
+                E[1] = {f.y, 0.0f};
+                E[2] = {f.z, 0.0f};
+            }
             if (cell >= 0) {
                 V3<float> F = antenna_vec<float>(p.rxa.kind, zeta_r, Rr, V3<float>{-d.x, -d.y, -d.z});
                 float re = F.x * E[0].re + F.y * E[1].re + F.z * E[2].re;
@@ -430,12 +434,32 @@ __device__ __forceinline__ void flush_ypr(float* g, int tx, float (&acc)[3]) {
     acc[0] = acc[1] = acc[2] = 0.0f;
 }
 
+#define RT_ROT_CACHE_VJP 16
+// Rotation of (yaw, pitch, roll) with its derivatives with respect to them.
+__device__ __forceinline__ Rot<Dual<3>> seeded_rot(const float* ypr) {
+    Dual<3> yaw = dconst<3>(ypr[0]), pitch = dconst<3>(ypr[1]), roll = dconst<3>(ypr[2]);
+    yaw.d[0] = 1.0f;
+    pitch.d[1] = 1.0f;
+    roll.d[2] = 1.0f;
+    return rot_ypr(yaw, pitch, roll);
+}
+
 template <int L, bool B = false>
 __global__ void __launch_bounds__(256) k_coverage_vjp(CovVjpParams q) {
     extern __shared__ float4 sm[];
     const CovParams& p = q.p;
-    stage_nodes(p.c, sm);
     typedef Dual<3> D3;
+    // each transmitter's rotation and its derivatives once per block
+    __shared__ D3 s_rot[RT_ROT_CACHE_VJP * 9];
+    const long long n_tx = p.c.total / (p.c.count > 0 ? p.c.count : 1);
+    const bool rot_cached = n_tx <= RT_ROT_CACHE_VJP;
+    if (rot_cached) {
+        for (int k = threadIdx.x; k < (int)n_tx; k += blockDim.x) {
+            const Rot<D3> R = seeded_rot(p.c.tx_ypr + 3 * k);
+            for (int i = 0; i < 9; i++) s_rot[9 * k + i] = R.m[i / 3][i % 3];
+        }
+    }
+    stage_nodes(p.c, sm);   // ends with a block barrier
     WarpFeed feed;
     bool alive = false;
     f3 o = mk(0, 0, 0), d = mk(0, 0, 1);
@@ -462,16 +486,6 @@ __global__ void __launch_bounds__(256) k_coverage_vjp(CovVjpParams q) {
             tx = next_tx;
             o = mk(p.c.tx_pos[3 * tx], p.c.tx_pos[3 * tx + 1], p.c.tx_pos[3 * tx + 2]);
             d = ray_dir(p.c, kd, i);
-            D3 yaw = dconst<3>(p.c.tx_ypr[3 * tx]), pitch = dconst<3>(p.c.tx_ypr[3 * tx + 1]),
-               roll = dconst<3>(p.c.tx_ypr[3 * tx + 2]);
-            yaw.d[0] = 1.0f;
-            pitch.d[1] = 1.0f;
-            roll.d[2] = 1.0f;
-            Rot<D3> Rt = rot_ypr(yaw, pitch, roll);
-            V3<D3> f = antenna_vec<D3>(p.txa.kind, zeta_t, Rt, v_const<D3>(d));
-            E[0] = {f.x, dconst<3>(0.0f)};
-            E[1] = {f.y, dconst<3>(0.0f)};
-            E[2] = {f.z, dconst<3>(0.0f)};
             last = -1;
             depth = 0;
             alive = true;
@@ -485,6 +499,18 @@ __global__ void __launch_bounds__(256) k_coverage_vjp(CovVjpParams q) {
         const bool more = depth < p.D;
         const long long cell = cov_segment_warp<false, L, B>(p, sm, alive, tx, o, d, last, more, id, t, cnt, cnt);
         if (alive) {
+            if (depth == 0 && (cell >= 0 || (more && id >= 0))) {   // as in k_coverage
+                Rot<D3> Rt;
+                if (rot_cached) {
+                    for (int q = 0; q < 9; q++) Rt.m[q / 3][q % 3] = s_rot[9 * tx + q];
+                } else {
+                    Rt = seeded_rot(p.c.tx_ypr + 3 * tx);
+                }
+                V3<D3> f = antenna_vec<D3>(p.txa.kind, zeta_t, Rt, v_const<D3>(d));
+                E[0] = {f.x, dconst<3>(0.0f)};
+                E[1] = {f.y, dconst<3>(0.0f)};
+                E[2] = {f.z, dconst<3>(0.0f)};
+            }
             if (cell >= 0) {
                 const float g = q.grad_gain[cell];
                 if (g != 0.0f) {
