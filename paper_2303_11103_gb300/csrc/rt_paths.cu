@@ -291,8 +291,9 @@ __global__ void __launch_bounds__(256) k_cand_prep(const uint64_t* __restrict__ 
                                                    KeyFmt f, const float* __restrict__ tx_pos,
                                                    const float4* __restrict__ planes, float* __restrict__ img,
                                                    const int32_t* __restrict__ rx_off, int n_tx, int n_rx,
-                                                   int64_t* cand_off, int64_t* work_off) {
+                                                   int64_t* cand_off, int64_t* work_off, unsigned long long* work) {
     const int64_t U = *Up;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *work = 0;   // the validation hands out its units here
     if (blockIdx.x == 0) cand_ranges(ck, U, f, rx_off, n_tx, n_rx, cand_off, work_off);
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < U; c += (int64_t)gridDim.x * blockDim.x)
         cand_img_one(ck, c, f, tx_pos, planes, img);
@@ -312,6 +313,7 @@ struct ValParams {
     int n_tx, n_rx;            // total work = work_off[n_tx]
     uint64_t* out;
     unsigned long long* count;
+    unsigned long long* work;   // units handed out (cleared before)
     long long cap;
     int n_sm;
     unsigned* status;
@@ -479,7 +481,14 @@ __device__ void validate_batch(const ValParams& p, const float4* sm, const ValWa
 // parameter in (0, 1)). Most pairs fail it; the ones that pass go to a
 // per-warp queue, and whenever 32 are queued they are validated in full
 // (validate_batch) with all lanes busy.
-template <bool C, int L>
+//
+// H: units are handed out in runs of 4 (a candidate against its receivers in
+// order) instead of dealt one by one. It pays where every warp gets many of
+// them: 32 transmitters x 250 receivers 277 us handed out, 374 dealt; 1 x 1000
+// receivers (24 units a warp) 95 and 75, since few runs do not spread the
+// receivers of the candidates that most pairs pass (line of sight, ground) over
+// the warps.
+template <bool C, int L, bool H = false>
 __global__ void __launch_bounds__(256, 4) k_validate(ValParams p) {
     extern __shared__ float4 sm[];
     const float4* src = node_base(p.s);
@@ -494,37 +503,8 @@ __global__ void __launch_bounds__(256, 4) k_validate(ValParams p) {
     const long long total = p.work_off[p.n_tx];   // warp units: (candidate, 32 receivers)
     TravCount cnt;
     int head = 0, count = 0;   // survivor queue (warp-uniform)
-    for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < total; u += wstride) {
-        // the unit's transmitter, candidate and first receiver (warp-uniform)
-        int lo = 0, hi = p.n_tx;  // largest t with work_off[t] <= u
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (p.work_off[mid] <= u) lo = mid; else hi = mid;
-        }
-        const int t = lo;
-        const long long R = p.rx_off ? (long long)(p.rx_off[t + 1] - p.rx_off[t]) : (long long)p.n_rx;
-        const long long chunks = (R + 31) >> 5;
-        const long long local = u - p.work_off[t];
-        const long long cl = local / chunks;
-        const long long r = ((local - cl * chunks) << 5) + lane;
-        const long long c = p.cand_off[t] + cl;
-        const uint64_t key = p.cand_key[c];
-        const int K = p.f.depth(key);
-        bool pass = false;
-        long long rxg = 0;
-        if (r < R) {
-            rxg = p.rx_off ? (long long)p.rx_off[t] + r : r;
-            f3 rx = mk(p.rx_pos[3 * rxg], p.rx_pos[3 * rxg + 1], p.rx_pos[3 * rxg + 2]);
-            if (K == 0) {
-                pass = true;
-            } else {
-                const float* img = p.cand_img + ((size_t)c * D + (K - 1)) * 3;
-                f3 dir = mk(img[0], img[1], img[2]) - rx;
-                const float4* tp = p.s.tris_o + 3 * (size_t)p.f.id(key, K - 1);
-                float th = tri_hit(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2), rx, dir);
-                pass = th > 0.0f && th < 1.0f;
-            }
-        }
+    // queues the lanes' survivors; a full batch is validated
+    auto take = [&](bool pass, long long c, long long rxg, int t) {
         const unsigned m = __ballot_sync(full, pass);
         if (pass) {
             const int e = (head + count + __popc(m & lt)) % VQ;
@@ -539,6 +519,115 @@ __global__ void __launch_bounds__(256, 4) k_validate(ValParams p) {
             head = (head + 32) % VQ;
             count -= 32;
             __syncwarp();
+        }
+    };
+    if (H) {
+        // the candidate and its last triangle are looked up once per run and candidate
+        constexpr int run = 4;
+        auto fetch = [&]() {
+            unsigned long long b = 0;
+            if (lane == 0) b = atomicAdd(p.work, (unsigned long long)run);
+            return (long long)__shfl_sync(full, b, 0);
+        };
+        long long u = fetch(), u_end = min(u + run, total);
+        bool moved = true;                          // another run
+        int t = 0, K = 0, chunk = 0, chunks = 0;   // chunk: the unit's 32 receivers
+        long long c = -1, c_end = 0, R = 0;
+        float4 q0, q1, q2;
+        f3 I = mk(0.0f, 0.0f, 0.0f);
+        q0 = q1 = q2 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        while (u < total) {
+            // the unit's transmitter, candidate and receivers (warp-uniform)
+            const bool fresh = moved || c >= c_end;
+            if (fresh) {
+                // units only rise: mostly this transmitter's or the next one's
+                if (p.work_off[t + 1] <= u) t++;
+                if (p.work_off[t + 1] <= u) {
+                    int hi = p.n_tx;   // largest t with work_off[t] <= u
+                    while (hi - t > 1) {
+                        const int mid = (t + hi) >> 1;
+                        if (p.work_off[mid] <= u) t = mid; else hi = mid;
+                    }
+                }
+                R = p.rx_off ? (long long)(p.rx_off[t + 1] - p.rx_off[t]) : (long long)p.n_rx;
+                chunks = (int)((R + 31) >> 5);
+                const long long local = u - p.work_off[t];
+                c = (local >> 32) ? local / chunks : (long long)((unsigned)local / (unsigned)chunks);
+                chunk = (int)(local - c * chunks);
+                c += p.cand_off[t];
+                c_end = p.cand_off[t + 1];
+                moved = false;
+            }
+            if (fresh || chunk == 0) {
+                const uint64_t key = p.cand_key[c];
+                K = p.f.depth(key);
+                if (K > 0) {
+                    const float* img = p.cand_img + ((size_t)c * D + (K - 1)) * 3;
+                    I = mk(img[0], img[1], img[2]);
+                    const float4* tp = p.s.tris_o + 3 * (size_t)p.f.id(key, K - 1);
+                    q0 = __ldg(tp);
+                    q1 = __ldg(tp + 1);
+                    q2 = __ldg(tp + 2);
+                }
+            }
+            const long long r = ((long long)chunk << 5) + lane;
+            const long long cand = c;
+            bool pass = false;
+            long long rxg = 0;
+            if (r < R) {
+                rxg = p.rx_off ? (long long)p.rx_off[t] + r : r;
+                pass = true;
+                if (K > 0) {
+                    const f3 rx = mk(p.rx_pos[3 * rxg], p.rx_pos[3 * rxg + 1], p.rx_pos[3 * rxg + 2]);
+                    const float th = tri_hit(q0, q1, q2, rx, I - rx);
+                    pass = th > 0.0f && th < 1.0f;
+                }
+            }
+            const int tx = t;
+            if (++chunk == chunks) {
+                chunk = 0;
+                c++;
+            }
+            if (++u == u_end) {
+                u = fetch();
+                u_end = min(u + run, total);
+                moved = true;
+            }
+            take(pass, cand, rxg, tx);
+        }
+    } else {
+        for (long long u = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < total; u += wstride) {
+            // the unit's transmitter, candidate and first receiver (warp-uniform)
+            int lo = 0, hi = p.n_tx;  // largest t with work_off[t] <= u
+            while (hi - lo > 1) {
+                int mid = (lo + hi) >> 1;
+                if (p.work_off[mid] <= u) lo = mid; else hi = mid;
+            }
+            const int t = lo;
+            const long long R = p.rx_off ? (long long)(p.rx_off[t + 1] - p.rx_off[t]) : (long long)p.n_rx;
+            const long long chunks = (R + 31) >> 5;
+            const long long local = u - p.work_off[t];
+            const long long cl = local / chunks;
+            const long long r = ((local - cl * chunks) << 5) + lane;
+            const long long c = p.cand_off[t] + cl;
+            const uint64_t key = p.cand_key[c];
+            const int K = p.f.depth(key);
+            bool pass = false;
+            long long rxg = 0;
+            if (r < R) {
+                rxg = p.rx_off ? (long long)p.rx_off[t] + r : r;
+                f3 rx = mk(p.rx_pos[3 * rxg], p.rx_pos[3 * rxg + 1], p.rx_pos[3 * rxg + 2]);
+                if (K == 0) {
+                    pass = true;
+                } else {
+                    const float* img = p.cand_img + ((size_t)c * D + (K - 1)) * 3;
+                    f3 dir = mk(img[0], img[1], img[2]) - rx;
+                    const float4* tp = p.s.tris_o + 3 * (size_t)p.f.id(key, K - 1);
+                    float th = tri_hit(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2), rx, dir);
+                    pass = th > 0.0f && th < 1.0f;
+                }
+            }
+            take(pass, c, rxg, t);
         }
     }
     if (count > 0) validate_batch<C, L>(p, sm, W, head, count, cnt);
@@ -712,6 +801,7 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
         return e != cudaSuccess ? e : cudaStreamSynchronize(st);
     };
     const uint32_t* Ud = nullptr;   // device candidate count
+    int64_t n_uniq = 0;             // the same, where the host has read it
     // hash table slots: a power of two, at least twice the keys
     auto slots_for = [](int64_t n) {
         int64_t S = 1024;
@@ -767,6 +857,7 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             RT_TRY(radix_sort64(ctx, bp<uint64_t>(ctx->keys_alt), bp<uint64_t>(ctx->cand_key),
                                 bp<uint32_t>(ctx->vals_alt), bp<uint32_t>(ctx->cand_wit), U, ctx->key_bits, true));
             Ud = cntp;
+            n_uniq = U;
         }
     }
     if (!use_hash) {
@@ -820,7 +911,7 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
     k_cand_prep<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((nkeys + 255) / 256, 8 * ctx->num_sms)), 256, 0, st>>>(
         bp<uint64_t>(ctx->cand_key), Ud, f, bp<float>(ctx->tx_pos), bp<float4>(ctx->planes), bp<float>(ctx->cand_img),
         ctx->rx_sets ? bp<int32_t>(ctx->rx_off_d) : nullptr, ctx->n_tx, ctx->n_rx, bp<int64_t>(ctx->cand_off),
-        bp<int64_t>(woffd));
+        bp<int64_t>(woffd), bp<unsigned long long>(ctx->counters) + RT_CNT_WORK);
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
     if (ctx->path_cap == 0) ctx->path_cap = 1 << 16;
@@ -829,7 +920,7 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
         RT_TRY(buf_reserve(ctx->path_key, sizeof(uint64_t) * ctx->path_cap));
         RT_TRY(buf_reserve(ctx->path_key_alt, sizeof(uint64_t) * ctx->path_cap));
         if (attempt > 0)
-            RT_TRY(cudaMemsetAsync(bp<unsigned long long>(ctx->counters) + RT_CNT_PATHS, 0, sizeof(unsigned long long), st));
+            RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, 2 * sizeof(unsigned long long), st));
         if (nkeys > 0 && n_pairs > 0) {
             ValParams vp;
             vp.s = dev_scene(ctx);
@@ -845,6 +936,7 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             vp.n_rx = ctx->n_rx;
             vp.out = bp<uint64_t>(ctx->path_key_alt);
             vp.count = bp<unsigned long long>(ctx->counters) + 1;
+            vp.work = bp<unsigned long long>(ctx->counters) + RT_CNT_WORK;
             vp.cap = ctx->path_cap;
             vp.n_sm = staged_nodes(ctx);
             vp.status = bp<unsigned>(ctx->status);
@@ -854,9 +946,15 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             RT_TRY(ensure_smem_attr((const void*)kern, smem));
             const int per_sm = blocks_per_sm((const void*)kern, 256, smem);
             // persistent grid: the work total is read on the device
-            const int64_t units = nkeys * std::max<int64_t>((n_pairs / std::max(ctx->n_tx, 1) + 31) / 32, 1);
+            const int64_t per_cand = std::max<int64_t>((n_pairs / std::max(ctx->n_tx, 1) + 31) / 32, 1);
+            const int64_t units = nkeys * per_cand;
             const int64_t need = (units + 7) / 8;   // 8 warps per block
             const int64_t grid = std::max<int64_t>(std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * ctx->num_sms), 1);
+            // every warp gets about 64 units (n_uniq: distinct candidates, where known)
+            if (!wide_layout(ctx) && !ctx->count_work && n_uniq * per_cand >= 64 * 8 * grid) {
+                kern = k_validate<false, 2, true>;
+                RT_TRY(ensure_smem_attr((const void*)kern, smem));
+            }
             prof_begin(ctx, "k_validate");
             kern<<<(unsigned)grid, 256, smem, st>>>(vp);
             prof_end(ctx);
