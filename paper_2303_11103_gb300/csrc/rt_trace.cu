@@ -19,7 +19,9 @@ namespace {
 // Key = place of the lattice direction along Hilbert curves over (phi, z),
 // three squares of 120 degrees by 2 (equal areas, nearly square in angle) of
 // 2^11 x 2^11 cells each: any run of rays in this order points into one patch
-// of directions (a Z-order curve jumps, and splits such a run in two).
+// of directions (a Z-order curve jumps, and splits such a run in two). The last
+// square is taken upside down, so that a trace ends with rays to the sky, the
+// shortest ones, and its warps end together.
 __global__ void k_perm_keys(long long N, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -29,6 +31,7 @@ __global__ void k_perm_keys(long long N, uint64_t* __restrict__ keys, uint32_t* 
     v = 3.0f * fminf(fmaxf(v, 0.0f), 0.99999f);
     const unsigned third = (unsigned)v;
     unsigned x = (unsigned)((v - (float)third) * 2048.0f), y = (unsigned)(u * 2048.0f);
+    if (third == 2) y = 2047u - y;
     unsigned code = third;
     // quadrant by quadrant from the top: (0,0), (0,1), (1,1), (1,0), the curve
     // inside the first mirrored in the diagonal and in the last in the other one
