@@ -479,10 +479,10 @@ ALU_PEAK_GOPS = 152 * 128 * 2.070
 # DRAM bytes (read + write) of one k_coverage launch of this workload, from
 # the ncu capture summarised in profiles/k_coverage_city_1e6rays.md; set to
 # None whenever the kernel changes until it is captured again.
-K_COVERAGE_TRAFFIC = 20.60e6
+K_COVERAGE_TRAFFIC = 21.33e6
 # L1/TEX throughput of the same launch (% of its peak, elapsed) and the
 # sector hit rate: the traversal's record reads are served by L1.
-K_COVERAGE_L1 = {"l1tex_throughput_pct": 61.3, "l1tex_sector_hit_pct": 85.9, "lts_throughput_pct": 2.8,
+K_COVERAGE_L1 = {"l1tex_throughput_pct": 31.1, "l1tex_sector_hit_pct": 88.5, "lts_throughput_pct": 3.4,
                  "source": "profiles/k_coverage_city_1e6rays.md (ncu --set full, one launch)"}
 
 
@@ -530,7 +530,8 @@ def roofline(name, rec, sbr_counts, cov_counts, hbm, src, probe):
             "bvh_width": BVH_WIDTH,
             "lane_count_gops": ALU_PEAK_GOPS, "frac_of_lane_count": ach / ALU_PEAK_GOPS,
             "ops_per_launch": ops, "ops_basis": f"{OPS_PER_NODE} per BVH node record ({BVH_WIDTH}-wide), "
-                                                f"{OPS_PER_TRI} per triangle record",
+                                                f"{OPS_PER_TRI} per triangle record, counted ray by ray "
+                                                "(the timed launch traces neighbouring rays as beams)",
             "requested_gbs": req_bytes / per_launch_s / 1e9, "hbm_peak_gbs": hbm, "hbm_peak_source": src,
             "ms_per_launch": per_launch_s * 1e3,
             "nodes_per_query": counts["nodes"] / max(queries(counts), 1),

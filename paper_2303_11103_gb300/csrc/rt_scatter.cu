@@ -175,7 +175,7 @@ __device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHit
 // the sum of dL/dg * g / S^2, times 2 S, goes to the hit's material (per block
 // in shared memory first).
 // Bound by the pairs no kept occluder answers and by the pairs' own
-// arithmetic. 1e5 rays x 1000 receivers in the city, mean of six sites: 1.37
+// arithmetic. 1e5 rays x 1000 receivers in the city, mean of six sites: 1.32
 // ms, where a thread per (ray, chunk of receivers) with a traversal per pair
 // took 3.83 ms. (One occluder kept instead of two: 7 % slower; the queued
 // segments as beams: 4 % slower, they fan out over the receivers.)
@@ -341,10 +341,12 @@ int scattering_impl(rt_ctx* ctx, int64_t N, float* gain, const float* up, float*
     // work units: up to SC_RAYS rays against a chunk of the receivers. The rays
     // of a unit share its occluders and its chunk's receivers amortise their
     // first hits, so both shrink only while the units would not fill the chip:
-    // to 128 rays and 32 receivers for 16 units per SM, to 32 rays and 4 receivers
-    // for one wave (2 x 1464 rays x 127 receivers: 0.10 ms; one thread per ray and
-    // 64 receivers took 1.22 ms). Below 16 receivers a unit is a warp's 32 rays
-    // (1e5 rays x 1 receiver: 51 us, blocks of four warps 62)
+    // to 128 rays and 32 receivers for 24 units per SM (city, 1000 receivers, mean
+    // of six sites: 16 units 1.41 ms, 24 1.32, 32 1.35, 48 1.44: first hits against
+    // the last wave's gap), to 32 rays and 4 receivers for one wave (2 x 1464 rays
+    // x 127 receivers: 0.10 ms; one thread per ray and 64 receivers took 1.22 ms).
+    // Below 16 receivers a unit is a warp's 32 rays (1e5 rays x 1 receiver: 51 us,
+    // blocks of four warps 62).
     int nr_max = ctx->n_rx;
     if (ctx->rx_sets) {
         nr_max = 0;
@@ -357,8 +359,8 @@ int scattering_impl(rt_ctx* ctx, int64_t N, float* gain, const float* up, float*
         return std::max<long long>(1, std::min<long long>(nr_max / receivers, (units + n_units(rays, 1) - 1) / n_units(rays, 1)));
     };
     p.rays = few ? 32 : SC_RAYS;
-    if (!few && n_units(p.rays, std::max(1, nr_max / 32)) < 16 * sms) p.rays = 128;
-    p.n_chunks = (int)chunks_for(p.rays, 16 * sms, 32);
+    if (!few && n_units(p.rays, std::max(1, nr_max / 32)) < 24 * sms) p.rays = 128;
+    p.n_chunks = (int)chunks_for(p.rays, 24 * sms, 32);
     if (n_units(p.rays, p.n_chunks) < wave) p.n_chunks = (int)chunks_for(p.rays, wave, 4);
     while (p.rays > 32 && n_units(p.rays, p.n_chunks) < wave) p.rays /= 2;
     const unsigned blocks = (unsigned)std::min<long long>(n_units(p.rays, p.n_chunks), 1ll << 30);
