@@ -5,8 +5,9 @@
 // Dense layers are tcgen05 GEMMs: BF16 operands staged in shared memory by
 // TMA (128-byte swizzle, 4-stage mbarrier pipeline), FP32 accumulators in
 // TMEM, one thread issuing MMAs, the four warps reading TMEM in the
-// epilogue (bias, ReLU, BF16 or FP32 store). Features, the 2-wide head, the
-// loss, transposes, column sums and Adam run on CUDA cores.
+// epilogue (bias, ReLU, BF16 or FP32 store). Inference and training run all
+// layers of a tile in one kernel each; the weight gradients of all layers are
+// one more, Adam another. Shapes those do not take go layer by layer.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
