@@ -256,7 +256,7 @@ int rt_destroy(rt_ctx* ctx) {
         buf_free(ctx->side_counters);
         buf_free(ctx->side_status);
     }
-    for (DevBuf* b : {&ctx->nodes, &ctx->pk, &ctx->tris, &ctx->tris_o, &ctx->planes, &ctx->planes64, &ctx->mat, &ctx->mats, &ctx->tx_pos,
+    for (DevBuf* b : {&ctx->nodes, &ctx->pk, &ctx->pk_order, &ctx->tris, &ctx->tris_o, &ctx->planes, &ctx->planes64, &ctx->mat, &ctx->mats, &ctx->tx_pos,
                       &ctx->tx_ypr, &ctx->rx_pos, &ctx->rx_ypr, &ctx->rx_off_d, &ctx->keys, &ctx->keys_alt,
                       &ctx->vals, &ctx->vals_alt, &ctx->ray_hits, &ctx->cand_key, &ctx->cand_wit, &ctx->cand_off,
                       &ctx->cand_img, &ctx->htab_key, &ctx->htab_wit, &ctx->htab_cnt, &ctx->dop_cyc, &ctx->arr_dirs,

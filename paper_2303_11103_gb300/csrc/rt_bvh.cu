@@ -895,11 +895,41 @@ float host_unord(unsigned u) {
 
 }  // namespace
 
+// Hilbert code of a leaf's centroid over axes ax and ay (origin lo, cells of
+// `cell`, 16 bits each), with the leaf's index.
+__global__ void k_pk_keys(const float4* __restrict__ tris, int n, int ax, int ay, float lox, float loy, float cell,
+                          uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const float4 v = tris[3 * (size_t)k], e1 = tris[3 * (size_t)k + 1], e2 = tris[3 * (size_t)k + 2];
+    const float c[3] = {v.x + (e1.x + e2.x) * (1.0f / 3.0f), v.y + (e1.y + e2.y) * (1.0f / 3.0f),
+                        v.z + (e1.z + e2.z) * (1.0f / 3.0f)};
+    unsigned x = (unsigned)fminf(fmaxf((c[ax] - lox) / cell, 0.0f), 65535.0f);
+    unsigned y = (unsigned)fminf(fmaxf((c[ay] - loy) / cell, 0.0f), 65535.0f);
+    uint64_t code = 0;
+    for (int b = 15; b >= 0; b--) {   // as in the ray order (rt_trace.cu)
+        const unsigned rx = (x >> b) & 1u, ry = (y >> b) & 1u;
+        code = (code << 2) | ((3u * rx) ^ ry);
+        if (ry == 0) {
+            if (rx) {
+                x = ~x;
+                y = ~y;
+            }
+            const unsigned t = x;
+            x = y;
+            y = t;
+        }
+    }
+    keys[k] = code;
+    vals[k] = (uint32_t)k;
+}
+
 // Boxes for traversal by beams (layout: rt_packet.cuh): a block takes 1024
 // consecutive leaves, a warp 32 of them; the block after the last set takes
 // the header, the large triangles and the padding. Every box is widened by
 // `margin`.
-__global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tris, int n, int n_big, float margin,
+__global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tris, const uint32_t* __restrict__ order,
+                                                   int n, int n_big, float margin,
                                                    int groups, int sets, float4* __restrict__ pk) {
     const int b0 = 0, b1 = 32 * groups, b2 = b1 + 32 * sets, bb = b2 + (sets + 31) / 32 * 32;   // first records
     const int records = bb + (n_big + 31) / 32 * 32;
@@ -940,9 +970,9 @@ __global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tr
         }
         return;
     }
-    const int g = 32 * blockIdx.x + w, k = 32 * g + lane;
-    leaf(k, k < n, b);
-    if (g < groups) put(b0 + k, b, k);
+    const int g = 32 * blockIdx.x + w, k = 32 * g + lane, t = order && k < n ? (int)order[k] : k;
+    leaf(t, k < n, b);
+    if (g < groups) put(b0 + k, b, t);
     auto reduce = [&]() {
         for (int q = 0; q < 3; q++)
             for (int o = 16; o > 0; o >>= 1) {
@@ -1222,8 +1252,30 @@ int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     RT_TRY(cudaGetLastError());
     const int groups = (n + 31) / 32, sets = (groups + 31) / 32;
     RT_TRY(buf_reserve(ctx->pk, 32 * (1 + 8 * 32 * ((size_t)groups + sets + (sets + 31) / 32 + (n_big + 31) / 32))));
+    // flat scenes: leaves along a Hilbert curve over the two long axes, whose runs
+    // of 32 are more compact than the Morton order's (city: 129 m of width and
+    // depth against 159)
+    const uint32_t* order = nullptr;
+    float lo[3], side[3];
+    for (int k = 0; k < 3; k++) {
+        lo[k] = host_unord(hi[k]);
+        side[k] = host_unord(hi[3 + k]) - lo[k];
+    }
+    const int thin = side[2] <= side[0] && side[2] <= side[1] ? 2 : side[1] <= side[0] ? 1 : 0;
+    const int ax = thin == 0 ? 1 : 0, ay = thin == 2 ? 1 : 2;
+    if (n > 32 && 4.0f * side[thin] <= std::min(side[ax], side[ay])) {
+        RT_TRY(buf_reserve(ctx->pk_order, (2 * sizeof(uint64_t) + 2 * sizeof(uint32_t)) * (size_t)n));
+        uint64_t *k0 = bp<uint64_t>(ctx->pk_order), *k1 = k0 + n;
+        uint32_t *v0 = reinterpret_cast<uint32_t*>(k1 + n), *v1 = v0 + n;
+        prof_begin(ctx, "k_pk_keys");
+        k_pk_keys<<<(n + B - 1) / B, B, 0, st>>>(bp<float4>(ctx->tris), n, ax, ay, lo[ax], lo[ay], ext / 65536.0f, k0, v0);
+        prof_end(ctx);
+        RT_TRY(cudaGetLastError());
+        RT_TRY(radix_sort64(ctx, k0, k1, v0, v1, n, 32));
+        order = v0;
+    }
     prof_begin(ctx, "k_pk_boxes");
-    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), n, (int)n_big, 4e-6f * ext, groups, sets,
+    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), order, n, (int)n_big, 4e-6f * ext, groups, sets,
                                           bp<float4>(ctx->pk));
     prof_end(ctx);
     RT_TRY(cudaGetLastError());

@@ -47,6 +47,7 @@ struct rt_ctx {
     int n_wnodes = 0;
     DevBuf planes64;   // [T*3] double2: FP64 unit normal and first vertex per triangle (original order)
     DevBuf pk;                 // boxes for traversal by beams (rt_packet.cuh)
+    DevBuf pk_order;           // build scratch: order of their leaves
 
     // devices
     int n_tx = 0, n_rx = 0;
