@@ -652,16 +652,16 @@ static TraceCommon make_common(rt_ctx* ctx, int64_t N, int64_t first, int64_t co
 
 // Whether a trace takes its rays as beams: on the binary layout, with no
 // traversal counts asked for, in the direction-coherent order, and from
-// PK_DENSITY rays per transmitter and triangle on. A warp's 32 rays then span
-// less than about a sixth of the spacing of the leaf groups at a quarter of the
-// scene's extent; wider beams meet more triangles than a ray's own traversal
-// does. City of 4802 triangles, 32 transmitters, depth 3, beams against single
-// rays: 2e4 rays each 401 / 238 us, 6e4 528 / 433, 2e5 957 / 1035; 4
-// transmitters of 1e6, map, 861 / 972; 770 triangles: 2e4 214 / 235, 6e4
-// 300 / 539.
+// `density` rays per transmitter and triangle on: PK_DENSITY, twice that for the
+// orientation gradient, whose rays carry twice the registers. Wider beams meet
+// more triangles than a ray's own traversal does. Beams against single rays (us):
+// 4802 triangles, path trace of 32 transmitters, depth 3, 2e4 rays each 456 / 240,
+// 6e4 451 / 433, 2e5 775 / 1024; map of 8 x 1e5 250 / 223, 4 x 1e6 702 / 939;
+// gradient of 2 x 3e5 278 / 240; 770 triangles: path trace 2e4 207 / 237, 6e4
+// 317 / 533, gradient of 4 x 1.5e4 208 / 146, 2 x 3e5 208 / 344.
 constexpr long long PK_DENSITY = 40;
-static bool use_beams(const rt_ctx* ctx, const TraceCommon& c) {
-    return !wide_layout(ctx) && !ctx->count_work && c.perm && ctx->n_tris > 0 && c.N >= PK_DENSITY * ctx->n_tris;
+static bool use_beams(const rt_ctx* ctx, const TraceCommon& c, long long density = PK_DENSITY) {
+    return !wide_layout(ctx) && !ctx->count_work && c.perm && ctx->n_tris > 0 && c.N >= density * ctx->n_tris;
 }
 
 // Shoot and bounce: appends every hit's candidate key with its position
@@ -776,7 +776,7 @@ int launch_coverage_vjp(rt_ctx* ctx, const rt_grid* g, int D, int64_t N, int tx_
     q.grad_ypr = grad_ypr;
     RT_TRY(cudaMemsetAsync(grad_ypr, 0, sizeof(float) * 3 * (size_t)ctx->n_tx, ctx->stream));
     size_t smem = staged_bytes(ctx);
-    auto kern = wide_layout(ctx) ? k_coverage_vjp<8> : use_beams(ctx, p.c) ? k_coverage_vjp<2, true> : k_coverage_vjp<2>;
+    auto kern = wide_layout(ctx) ? k_coverage_vjp<8> : use_beams(ctx, p.c, 2 * PK_DENSITY) ? k_coverage_vjp<2, true> : k_coverage_vjp<2>;
     RT_TRY(ensure_smem_attr((const void*)kern, smem));
     RT_TRY(cudaMemsetAsync(ctx->counters.p, 0, sizeof(unsigned long long), ctx->stream));
     int grid = trace_grid(ctx, (const void*)kern, smem);
