@@ -2,7 +2,8 @@
 // together go through the scene as one beam.
 //
 // Besides the binary hierarchy the scene has an implicit tree of 32 children a
-// node: groups of 32 consecutive leaves (Morton order), sets of 32 groups; the
+// node: groups of 32 leaves (along a Hilbert curve in flat scenes, else in
+// Morton order), sets of 32 groups; the
 // large triangles stand apart, 32 a round. A lane tests one child's box
 // against the beam (the interval of the rays' origins moving with the interval
 // of their directions), so one round answers for 32 boxes and all rays of the
