@@ -97,3 +97,35 @@ def test_segment_beams_find_the_same_paths(nx, ny):
     assert len(pa["wedge"]) > 0
     assert np.array_equal(ga != 0, gb != 0)
     assert np.allclose(ga, gb, rtol=1e-4, atol=1e-6 * max(gb.max(), 1e-30))
+
+
+@pytest.mark.parametrize("n_rx,sets", [(2000, False), (1999, True)])
+def test_handed_out_validation_units(n_rx, sets):
+    """Enough candidates and receivers that the validation hands its units out in
+    runs (the binary layout), against units dealt one by one (8-wide): the same
+    paths, also with uneven receiver sets (one empty, ragged last units)."""
+    sc = _city(8)
+    rng = np.random.default_rng(n_rx)
+    n_tx = 8
+    pos = np.concatenate([rng.uniform(-80.0, 80.0, (n_tx, 2)), rng.uniform(30.0, 60.0, (n_tx, 1))], 1).astype(np.float32)
+    cut = np.array([0, 3000, 3000, 5001, 9000, 9001, 12000, 14000, 15990]) if sets else None
+    n = int(cut[-1]) if sets else n_rx
+    rx = np.concatenate([rng.uniform(-95.0, 95.0, (n, 2)), np.full((n, 1), 1.5)], 1).astype(np.float32)
+    out = []
+    for width in (2, 8):
+        tr = rt.Tracer(0, FC)
+        try:
+            tr.set_bvh_width(width)
+            tr.load_scene(sc)
+            tr.set_tx(pos, np.zeros((n_tx, 3), np.float32), S.V_ISO)
+            tr.set_rx(rx, np.zeros((n, 3), np.float32), S.V_ISO, None if cut is None else [int(v) for v in cut])
+            tr.compute_paths(3, 200000)
+            out.append({k: v.cpu().numpy() for k, v in tr.paths().items()})
+            units = len(tr.candidates()[0]) * ((n if not sets else n // n_tx) + 31) // 32
+        finally:
+            tr.close()
+    assert units >= 64 * 8 * 608   # what the rule asks for at 4 blocks on 152 SMs
+    a, b = out
+    assert len(a["depth"]) > 1000
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
