@@ -834,12 +834,18 @@ __global__ void __launch_bounds__(FM_THREADS, 1) k_mlp_fused(const __grid_consta
 // bits). Roles:
 //   warps 0-7   features, then every pass's epilogue: chunk c by warps
 //               4 (c & 1) .. + 3, so that the next pass starts on chunk 0 while
-//               chunks 2 and 3 are still in TMEM;
+//               chunks 2 and 3 are still in TMEM (W = 64: each four warps take
+//               half of the columns of the one chunk);
 //   warp 8      streams the weights by TMA, W and later W^T, in 64-column chunks;
 //   warp 9      issues tcgen05.mma (M 128, N W, K 16) chunk by chunk;
 //   warp 10     stores every finished chunk.
 // Values are those of the layer-by-layer kernels bit for bit (same MMA shapes
-// and order, same sums in the head and the loss). Every wait is bounded; after
+// and order, same sums in the head and the loss). A wait by parity tells a phase
+// from the one after it, not from the next but one, so no barrier completes a
+// second phase before every waiter has seen the first: warps 0-7 all arrive in
+// each pass after their own waits, and the chunks that are only stored (H_L and
+// dZ_0) have barriers that warp 10 alone waits on, since warp 9 holds up nothing
+// between them and the chunks after them. Every wait is bounded; after
 // a timeout the roles run on without waiting, on the same control flow.
 // One tile per CTA: 128 CTAs at B = 16384, and the per-pass latency (first
 // chunk's epilogue + four chunks of MMA) bounds it: 67 us for B = 16384,
@@ -875,8 +881,8 @@ struct TrainLayout {
         dy = (bf + 4u * (uint32_t)(6 * F + 12) + 7u) & ~7u;
         bars = dy + 128u * 8u;
     }
-    // ring full / empty, chunks ready, features ready, MMA done, stored, drain
-    __host__ __device__ uint32_t bytes(int NS) const { return bars + 8u * (2 * NS + 4 + 4); }
+    // ring full / empty, chunks ready, chunks ready to be stored only, features ready, MMA done, stored, drain
+    __host__ __device__ uint32_t bytes(int NS) const { return bars + 8u * (2 * NS + 4 + 4 + 4); }
 };
 
 __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_constant__ TrainMaps maps, TrainArgs a) {
@@ -894,8 +900,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
     float2* s_dy = (float2*)(base + lay.dy);
     uint64_t* bars = (uint64_t*)(base + lay.bars);
     const uint32_t full0 = su32(bars), empty0 = su32(bars + NS), chunk0 = su32(bars + 2 * NS);
-    const uint32_t feat = su32(bars + 2 * NS + 4), done = su32(bars + 2 * NS + 5), stored = su32(bars + 2 * NS + 6);
-    const uint32_t drain = su32(bars + 2 * NS + 7);
+    const uint32_t only0 = su32(bars + 2 * NS + 4);
+    const uint32_t feat = su32(bars + 2 * NS + 8), done = su32(bars + 2 * NS + 9), stored = su32(bars + 2 * NS + 10);
+    const uint32_t drain = su32(bars + 2 * NS + 11);
     const uint32_t slot_bytes = (uint32_t)W * 128u;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < L * W; i += TC_THREADS) {
@@ -919,7 +926,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
             mbar_init(full0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, 1);
         }
-        for (int c = 0; c < 4; c++) mbar_init(chunk0 + 8 * c, 128);
+        for (int c = 0; c < 4; c++) {
+            mbar_init(chunk0 + 8 * c, nc == 1 ? 256 : 128);
+            mbar_init(only0 + 8 * c, nc == 1 ? 256 : 128);
+        }
         mbar_init(feat, 256);
         mbar_init(done, 1);
         mbar_init(stored, 1);
@@ -965,9 +975,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
                 for (int p = 0; p < passes; p++, pass++) {
                     const int nk = p == 0 ? nc0 : nc;
                     if (p == 0) wait(feat, ft);
-                    if (p == L)   // the last hidden output is no MMA's input
-                        for (int c = 0; c < nc; c++) wait(chunk0 + 8 * c, stage);
-                    if (p == L) stage++;
                     for (int kc = 0; kc < nk; kc++, it++) {
                         const uint32_t s = it % NS;
                         if (p > 0) wait(chunk0 + 8 * kc, stage);
@@ -983,14 +990,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
                     }
                     mma_commit(done);
                     if (p > 0) stage++;
-                    if (p == passes - 1) {   // dZ_0 (H_1 when there is one layer) is only stored
-                        for (int c = 0; c < nc; c++) wait(chunk0 + 8 * c, stage);
-                        stage++;
-                        if (L == 1) {
-                            for (int c = 0; c < nc; c++) wait(chunk0 + 8 * c, stage);
-                            stage++;
-                        }
-                    }
                 }
             // every MMA issued has completed before TMEM is released
             mma_commit(drain);
@@ -998,19 +997,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
         }
     } else if (warp == 10) {
         if (lane == 0) {
-            uint32_t ft = 0, stage = 0;
+            uint32_t ft = 0, stage = 0, only = 0;   // tiles, phases of the two kinds of chunk barriers
             for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ft++)
                 for (int q = 0; q <= 2 * L; q++) {   // features, H_1 .. H_L, dZ_{L-1} .. dZ_0
                     const CUtensorMap* mp = q == 0 ? &maps.h0 : q <= L ? &maps.h : &maps.z;
                     const int64_t r0 = q == 0 ? 0 : q <= L ? (int64_t)(q - 1) * a.cap : (int64_t)(2 * L - q) * a.cap;
                     const int nk = q == 0 ? nc0 : nc;
+                    const bool last = q == L || q == 2 * L;   // H_L, dZ_0: no MMA's input
                     if (q == 0) wait(feat, ft);
                     for (int c = 0; c < nk; c++) {
-                        if (q > 0) wait(chunk0 + 8 * c, stage);
+                        if (q > 0) wait((last ? only0 : chunk0) + 8 * c, last ? only : stage);
                         if (!abort_flag)
                             tma_store_2d(mp, su32(act + c * 16384), c * 64, (int)(r0 + (int64_t)tile * 128));
                     }
-                    if (q > 0) stage++;
+                    if (last) only++;
+                    else if (q > 0) stage++;
                     bulk_commit();
                     bulk_wait_read0();
                     mbar_arrive(stored);
@@ -1020,6 +1021,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
     } else {
         const int g = warp >> 2, row = (warp & 3) * 32 + lane;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        const int c_first = nc == 1 ? 0 : g;
         uint32_t nst = 0, pass = 0;   // store phases and passes so far
         for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
             const int64_t q = (int64_t)tile * 128 + row;
@@ -1055,13 +1057,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
                 nst++;
                 // bits of H_{l+1} > 0 written forward; those of H_l applied backward
                 uint32_t* mk = s_mask + (size_t)(fwd ? l : l - 1) * (W / 32) * 128 + row;
-                for (int c = g; c < nc; c += 2) {
+                const uint32_t ready = p == L - 1 || p == passes - 1 ? only0 : chunk0;
+                for (int c = c_first; c < nc; c += 2) {
                     uint32_t r2[2][32];
                     tmem_ld32(acc + (uint32_t)c * 64u, r2[0]);
                     tmem_ld32(acc + (uint32_t)c * 64u + 32u, r2[1]);
                     tmem_wait_ld();
 #pragma unroll
                     for (int hh = 0; hh < 2; hh++) {
+                        if (nc == 1 && hh != g) continue;
                         uint32_t packed[16];
                         const int c0 = 64 * c + 32 * hh;
                         if (fwd) {
@@ -1098,7 +1102,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
                     }
                     fence_async_smem();
                     tc_fence_before();
-                    mbar_arrive(chunk0 + 8 * c);
+                    mbar_arrive(ready + 8 * c);
                 }
                 if (p != L - 1) continue;
                 // the head, the loss and their gradients
@@ -1166,9 +1170,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
                 wait(stored, nst - 1);
                 nst++;
                 const float2 d = s_dy[row];
-                for (int c = g; c < nc; c += 2) {
+                for (int c = c_first; c < nc; c += 2) {
 #pragma unroll
                     for (int hh = 0; hh < 2; hh++) {
+                        if (nc == 1 && hh != g) continue;
                         const int c0 = 64 * c + 32 * hh;
                         const uint32_t bits = mk[(2 * c + hh) * 128];
 #pragma unroll
@@ -1186,7 +1191,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_train_chain(const __grid_cons
                     }
                     fence_async_smem();
                     tc_fence_before();
-                    mbar_arrive(chunk0 + 8 * c);
+                    mbar_arrive((L == 1 ? only0 : chunk0) + 8 * c);
                 }
             }
         }

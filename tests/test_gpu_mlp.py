@@ -182,3 +182,13 @@ def test_train_step_shapes(F, W, L, B, first):
             assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b) + 1e-12, (l, n)
             o += n
     S.close()
+
+
+@pytest.mark.parametrize("F,W,L,B", [(32, 64, 3, 128),          # one chunk of columns, both groups of warps on it
+                                     (32, 64, 2, 128 * 153),    # the same over a second tile
+                                     (64, 64, 8, 256),
+                                     (32, 128, 1, 128 * 153),   # one layer, a second tile
+                                     (32, 256, 1, 128)])
+def test_train_step_chunks(F, W, L, B):
+    """One fused step where warps share a chunk or two stored-only chunks follow each other."""
+    test_train_step_shapes(F, W, L, B, 0)
