@@ -106,6 +106,9 @@ def _train(sur, x, t, epochs, batch, lr, lr_end, seed):
             sur.train_step(xe[b * batch:(b + 1) * batch], te[b * batch:(b + 1) * batch], cur, acc)
             k += 1
         losses.append(float(acc.item()) / (n // batch))
+        # a step whose kernel gave up a wait has trained on unfinished gradients
+        if sur.status():
+            raise rt.RtError(-5, "a training kernel gave up a wait: the parameters are not usable")
     return losses
 
 
