@@ -1,5 +1,7 @@
 // rt_api.cu -- the C ABI (include/rt.h): context, argument checks, buffer
 // ownership and error reporting around the kernels.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -65,6 +67,7 @@ int set_err(rt_ctx* ctx, int code, const std::string& msg) {
 
 int set_cuda(rt_ctx* ctx, cudaError_t e, const char* what) {
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
+    cudaGetLastError();   // reported here, not again by the next launch's check
     return set_err(ctx, e == cudaErrorMemoryAllocation ? RT_ERR_OOM : RT_ERR_CUDA, m);
 }
 
@@ -123,6 +126,31 @@ int blocks_per_sm(const void* kernel, int block, size_t smem) {
     }
     done[key] = n;
     return n;
+}
+
+bool device_range(const rt_ctx* ctx, const void* p, size_t bytes) {
+    typedef CUresult (*GetAttributes)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const GetAttributes get = []() -> GetAttributes {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return (GetAttributes)fn;
+    }();
+    if (!get) return false;
+    CUmemorytype type = (CUmemorytype)0;
+    int dev = -1;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[4] = {&type, &dev, &base, &size};
+    const CUdeviceptr a = (CUdeviceptr)(uintptr_t)p;
+    return get(4, what, out, a) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && dev == ctx->device && base <= a &&
+           a - base <= size && bytes <= size - (a - base);
 }
 
 void prof_begin(rt_ctx* ctx, const char* name) {
@@ -521,7 +549,8 @@ int rt_get_paths(rt_ctx* ctx, int64_t* offsets, int32_t* seq, float* points, int
         {length, &ctx->path_len, sizeof(double) * (size_t)P}};
     for (const auto& a : arrays) {
         if (!a.dst || a.bytes == 0) continue;
-        if (a.bytes > a.src->bytes || (uintptr_t)a.dst % 4) {   // not computed for these devices, or not on a word boundary
+        // not computed for these devices, not on a word boundary, or not a kernel's to write
+        if (a.bytes > a.src->bytes || (uintptr_t)a.dst % 4 || !device_range(ctx, a.dst, a.bytes)) {
             RT_TRY(cudaMemcpyAsync(a.dst, a.src->p, a.bytes, cudaMemcpyDeviceToDevice, st));
             continue;
         }

@@ -548,6 +548,11 @@ template <int NP>
 cudaError_t launch_freq(rt_ctx* ctx, const int64_t* off, const float* a, const float* tau, const double* freqs,
                         int K, float* H, int64_t n_pairs) {
     dim3 grid((unsigned)n_pairs, (unsigned)((K + HF_THREADS * HF_RUN - 1) / (HF_THREADS * HF_RUN)));
+    const size_t bytes = sizeof(float2) * NP * (size_t)K * (size_t)n_pairs;
+    if (!device_range(ctx, H, bytes)) {   // refused here unless a kernel can write it all the same
+        const cudaError_t e = cudaMemsetAsync(H, 0, bytes, ctx->stream);
+        if (e != cudaSuccess) return e;
+    }
     prof_begin(ctx, "k_freq");
     k_freq<NP><<<grid, HF_THREADS, 0, ctx->stream>>>(off, (const float2*)a, tau, freqs, K, (float2*)H);
     prof_end(ctx);

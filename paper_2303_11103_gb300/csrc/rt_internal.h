@@ -147,6 +147,11 @@ struct rt_ctx {
 // least `bytes` (the attribute call is made once per kernel, device and size
 // increase; thread-safe).
 cudaError_t ensure_smem_attr(const void* kernel, size_t bytes);
+// Whether [p, p + bytes) lies in one allocation on the context's device. A
+// kernel may write there; other destinations (host memory, another device's,
+// a buffer too small) go through cudaMemcpyAsync or cudaMemsetAsync, which
+// take or refuse them.
+bool device_range(const rt_ctx* ctx, const void* p, size_t bytes);
 // resident blocks per SM of kernel at (block, dynamic shared memory), cached per device
 int blocks_per_sm(const void* kernel, int block, size_t smem);
 
