@@ -1058,7 +1058,14 @@ int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     if (!(ext > 0.0f)) ext = 1.0f;
     ctx->extent = ext;
     ctx->tmin = 2e-6f * ext;
-    const float pad = 1e-6f * ext;
+    // Boxes are widened beyond what rounding can shift a hit. Plane distances are
+    // rounded in proportion to the coordinates and the distance from the ray's
+    // origin (three roundings of 2^-24), so the margins go by the largest
+    // coordinate where that exceeds the extent (a scene in map coordinates); they
+    // hold for origins up to four times as far out.
+    float scale = ext;
+    for (int k = 0; k < 6; k++) scale = std::max(scale, std::fabs(host_unord(hi[k])));
+    const float pad = 1e-6f * scale;
     // sorted order: triangles of the hierarchy (Morton order), then the large ones (id order)
     const unsigned n_big = hi[12];
     const int n = T - (int)n_big;
@@ -1275,7 +1282,7 @@ int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
         order = v0;
     }
     prof_begin(ctx, "k_pk_boxes");
-    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), order, n, (int)n_big, 4e-6f * ext, groups, sets,
+    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), order, n, (int)n_big, 4e-6f * scale, groups, sets,
                                           bp<float4>(ctx->pk));
     prof_end(ctx);
     RT_TRY(cudaGetLastError());

@@ -500,7 +500,8 @@ __device__ __forceinline__ bool any_hit_b(const DevScene& s, const float4* sm, i
 
 // Whether the triangle `ref` (from an earlier any_hit_b) occludes this
 // segment: one triangle test instead of a traversal. The traversal would find
-// it too: a leaf's box is padded beyond what rounding can shift a hit.
+// it too: a leaf's box is padded beyond what rounding can shift a hit (origins
+// within four times the scene's extent or largest coordinate: rt_bvh.cu).
 __device__ __forceinline__ bool ref_hit(const DevScene& s, int ref, f3 o, f3 d, float tmax, int ex0, int ex1) {
     if (ref == RT_NO_REF) return false;
     const float4* tp = s.tris + 3 * (size_t)ref;

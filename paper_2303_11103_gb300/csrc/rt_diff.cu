@@ -139,7 +139,9 @@ constexpr int DF_Q = 64;   // entries of a warp's queues
 // Whether some cell of a grid tile may have its Keller point on the edge
 // (0 < t < len): t = ts + (tr - ts) rs / (rs + rr) for the extremes of tr
 // (place along the edge) and rr (distance from it) over the tile, which lies
-// within `rad` of its centre, widened by far more than rounding.
+// within `rad` of its centre, widened by far more than rounding: `rad` reaches
+// to the tile's corners, two thirds of a cell beyond its outermost centres,
+// which covers the rounding of far coordinates for cells of a few float steps.
 __device__ __forceinline__ bool tile_reached(const CellGrid& g, int tile, int tiles_y, f3 A, f3 e, float len, float ts,
                                              float rs) {
     const int cx = tile / tiles_y, cy = tile - cx * tiles_y;

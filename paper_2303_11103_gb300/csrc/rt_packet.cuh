@@ -11,9 +11,10 @@
 // are taken nearest first while they begin before the farthest current hit;
 // triangles that the beam reaches are tested by every ray, with the per-ray
 // traversal's test and ties, so both find the same hits: a hit is the smallest
-// distance over all triangles, equal ones to the lowest id, and the beam's
-// boxes are widened (4e-6 of the scene's extent) beyond what rounding can
-// shift.
+// distance over all triangles, equal ones to the lowest id, and the boxes are
+// widened beyond what rounding can shift: by 4e-6 of the scene's extent or of
+// its largest coordinate, where a plane at p seen from o is off by at most
+// 3.6e-7 (|p| + |o|) (rounded products and a reciprocal within two units).
 //
 // Boxes at s.pk, 32-byte records: first (groups, sets, large triangles rounded
 // up to 32, records of a copy), then 8 copies, one for each octant of
