@@ -37,10 +37,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 }
 
 // C[M x N] = act(A[M x K] B[N x K]^T + bias), A and B BF16 row-major (K
-// contiguous), C FP32 or BF16 row-major with leading dimension ldc. mask
-// (optional, BF16 [M x N], same leading dimension): C is zero where it is not
-// positive, the derivative of the ReLU that produced it.
-template <int BN>
+// contiguous), C FP32 or BF16 row-major with leading dimension ldc. MASK: C is
+// zero where mask (BF16 [M x N], same leading dimension) is not positive, the
+// derivative of the ReLU that produced it (a variant of its own: as a test of
+// the pointer it cost every layer of a forward pass 2 to 4 us).
+template <int BN, bool MASK>
 __global__ void __launch_bounds__(128, 1) k_gemm(const __grid_constant__ CUtensorMap ta,
                                                   const __grid_constant__ CUtensorMap tb, int M, int N, int K,
                                                   const float* __restrict__ bias, int relu, int out_bf16,
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(128, 1) k_gemm(const __grid_constant__ CUtenso
                 if (relu) x = fmaxf(x, 0.0f);
                 v[j] = x;
             }
-            if (mask) {
+            if (MASK) {
                 const __nv_bfloat16* mp = mask + (size_t)row * ldc + col;
                 if (col + 32 <= N) {
 #pragma unroll
@@ -1243,16 +1244,23 @@ size_t gemm_smem() {
     return (size_t)GSTAGES * (GM * GK * 2 + BN * GK * 2) + 1024;
 }
 
+template <int BN, bool MASK>
+cudaError_t launch_gemm_m(cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K,
+                          const float* bias, int relu, int out_bf16, void* C, int ldc, const void* mask,
+                          unsigned* err) {
+    size_t smem = gemm_smem<BN>();
+    cudaError_t e = ensure_smem_attr((const void*)k_gemm<BN, MASK>, smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((unsigned)((M + GM - 1) / GM), (unsigned)((N + BN - 1) / BN));
+    k_gemm<BN, MASK><<<grid, 128, smem, st>>>(ta, tb, M, N, K, bias, relu, out_bf16, C, ldc, (const __nv_bfloat16*)mask, err);
+    return cudaGetLastError();
+}
 template <int BN>
 cudaError_t launch_gemm_t(cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K,
                           const float* bias, int relu, int out_bf16, void* C, int ldc, const void* mask,
                           unsigned* err) {
-    size_t smem = gemm_smem<BN>();
-    cudaError_t e = ensure_smem_attr((const void*)k_gemm<BN>, smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((M + GM - 1) / GM), (unsigned)((N + BN - 1) / BN));
-    k_gemm<BN><<<grid, 128, smem, st>>>(ta, tb, M, N, K, bias, relu, out_bf16, C, ldc, (const __nv_bfloat16*)mask, err);
-    return cudaGetLastError();
+    return (mask ? launch_gemm_m<BN, true> : launch_gemm_m<BN, false>)(st, ta, tb, M, N, K, bias, relu, out_bf16, C, ldc,
+                                                                       mask, err);
 }
 
 }  // namespace
