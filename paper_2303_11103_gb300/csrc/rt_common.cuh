@@ -291,6 +291,13 @@ __device__ __forceinline__ int wide_ref(const float4* np, int slot) {
     return reinterpret_cast<const int*>(np + 12)[slot];
 }
 
+// a / b for 0 <= a, 0 < b: in 32 bits where both fit, about a fifth of the
+// 64-bit division's instructions.
+__device__ __forceinline__ long long div_ll(long long a, long long b) {
+    if (((a | b) >> 32) == 0) return (unsigned)a / (unsigned)b;
+    return a / b;
+}
+
 // Per-lane traversal counters (BVH node records and triangle records
 // fetched, queries), flushed once per warp at kernel end.
 struct TravCount {

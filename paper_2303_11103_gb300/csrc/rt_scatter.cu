@@ -73,23 +73,22 @@ __device__ float directive_norm(int alpha, float ci) {
     return ldexpf(tot, -alpha);
 }
 
-// Rays of a work unit at most, entries of a warp's queue.
-constexpr int SC_RAYS = 256, SC_Q = 64;
+// Rays of a work unit at most, warps of its block, entries of a warp's queue.
+constexpr int SC_RAYS = 256, SC_WARPS = 4, SC_Q = 64;
 
-// A unit's scattering hits (RAYS at most), in shared memory.
-template <int RAYS>
+// A unit's scattering hits, in shared memory.
 struct ScatHits {
-    float4 pt[RAYS];    // hit point, hit triangle
-    float4 nm[RAYS];    // normal on the side the ray came from, material
-    float4 tx[RAYS];    // transmit power of both ports, coefficient S, pattern exponent
-    float4 dir[RAYS];   // specular direction, F_alpha / pi (directive patterns only)
+    float4 pt[SC_RAYS];    // hit point, hit triangle
+    float4 nm[SC_RAYS];    // normal on the side the ray came from, material
+    float4 tx[SC_RAYS];    // transmit power of both ports, coefficient S, pattern exponent
+    float4 dir[SC_RAYS];   // specular direction, F_alpha / pi (directive patterns only)
 };
 
 // Any occluder between a queued (hit, receiver) pair, then its contribution:
 // lane < take handles entry n + lane. Called by all 32 lanes; the occluder
 // found last goes to ref0, the one before it to ref1.
-template <bool VJP, int LY, int RAYS>
-__device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHits<RAYS>& h, const int* qr,
+template <bool VJP, int LY>
+__device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHits& h, const int* qr,
                                               const uint16_t* qh, int n, int take, int t, float* sgrad, int& ref0,
                                               int& ref1, TravCount& cnt) {
     const unsigned full = 0xffffffffu;
@@ -179,14 +178,11 @@ __device__ __forceinline__ void scatter_batch(const ScatParams& p, const ScatHit
 // ms, where a thread per (ray, chunk of receivers) with a traversal per pair
 // took 3.83 ms. (One occluder kept instead of two: 7 % slower; the queued
 // segments as beams: 4 % slower, they fan out over the receivers.)
-// W: warps of a block; 4, or 1 (with 32 rays a unit) where the receivers are few
-// and the first hits weigh as much as the pairs, so that no warp waits for
-// another's rays.
-template <bool VJP, int LY, int W>
-__global__ void __launch_bounds__(32 * W, W == 4 ? 7 : 28) k_scatter(ScatParams p) {
-    constexpr int RAYS = W == 1 ? 32 : SC_RAYS;
+template <bool VJP, int LY>
+__global__ void __launch_bounds__(32 * SC_WARPS, 7) k_scatter(ScatParams p) {
+    constexpr int W = SC_WARPS;
     extern __shared__ float sgrad[];
-    __shared__ ScatHits<RAYS> h;
+    __shared__ ScatHits h;
     __shared__ int q_rx[W][SC_Q];
     __shared__ uint16_t q_hit[W][SC_Q];
     __shared__ int n_hit;
@@ -199,9 +195,9 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 7 : 28) k_scatter(ScatParams 
     TravCount cnt;
     int ref0 = RT_NO_REF, ref1 = RT_NO_REF;   // the last two occluders of recent pairs
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-        const long long tb = u / p.n_chunks;
+        const long long tb = div_ll(u, p.n_chunks);
         const int chunk = (int)(u - tb * p.n_chunks);
-        const int t = (int)(tb / batches);
+        const int t = (int)div_ll(tb, batches);
         const long long i0 = (tb - (long long)t * batches) * p.rays;
         // this chunk of the transmitter's receivers
         const int rb0 = p.rx_off ? p.rx_off[t] : 0, re0 = p.rx_off ? p.rx_off[t + 1] : p.n_rx;
@@ -261,7 +257,8 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 7 : 28) k_scatter(ScatParams 
         const int nt = (nh + 31) / 32;
         const long long steps = (long long)(re - rb) * nt;
         const long long step0 = steps * wp / W, step1 = steps * (wp + 1) / W;
-        int r = nt ? rb + (int)(step0 / nt) : rb, tile = nt ? (int)(step0 % nt) : 0;
+        const int r0 = nt ? (int)div_ll(step0, nt) : 0;
+        int r = rb + r0, tile = (int)(step0 - (long long)r0 * nt);
         f3 rx = mk(0, 0, 0);
         for (long long step = step0; step < step1; step++) {
             if (step == step0 || tile == 0) rx = mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
@@ -284,16 +281,118 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 7 : 28) k_scatter(ScatParams 
             }
             nq += __popc(om);
             __syncwarp();
-            if (nq >= 32) {
-                nq -= 32;
-                scatter_batch<VJP, LY, RAYS>(p, h, q_rx[wp], q_hit[wp], nq, 32, t, sgrad, ref0, ref1, cnt);
+            // 32 of them, or what is left at the end (one call: a second copy of the
+            // traversal costs a cold instruction cache 2 to 4 us)
+            while (nq >= 32 || (step + 1 == step1 && nq > 0)) {
+                const int take = min(nq, 32);
+                nq -= take;
+                scatter_batch<VJP, LY>(p, h, q_rx[wp], q_hit[wp], nq, take, t, sgrad, ref0, ref1, cnt);
             }
             if (++tile == nt) {
                 tile = 0;
                 r++;
             }
         }
-        if (nq > 0) scatter_batch<VJP, LY, RAYS>(p, h, q_rx[wp], q_hit[wp], 0, nq, t, sgrad, ref0, ref1, cnt);
+    }
+    if (VJP && p.grad_smem) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < p.n_mat; i += blockDim.x)
+            if (sgrad[i] != 0.0f) atomicAdd(p.grad + i, sgrad[i]);
+    }
+}
+
+
+// The same for few receivers, where the first hits weigh more than the pairs:
+// a thread a ray, which keeps its hit in registers and takes every receiver of
+// its transmitter in turn; the warp's lanes visit the same receiver together and
+// add up their contributions with one atomic when they share the transmitter.
+// Nothing is packed or queued, so one chain of first hit, segment and sum bounds
+// it: 1e5 rays x 1 receiver 60 us, k_scatter 63. VJP: each ray's sum of
+// dL/dg * g / S^2 goes, times 2 S, to its material.
+template <bool VJP, int LY>
+__global__ void __launch_bounds__(128) k_scatter_few(ScatParams p) {
+    extern __shared__ float sgrad[];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    if (VJP && p.grad_smem) {
+        for (int i = threadIdx.x; i < p.n_mat; i += blockDim.x) sgrad[i] = 0.0f;
+        __syncthreads();
+    }
+    const long long total = (long long)p.n_tx * p.N, step = (long long)gridDim.x * blockDim.x;
+    TravCount cnt;
+    for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; b < total; b += step) {
+        const bool in = b + lane < total;
+        const long long slot = in ? b + lane : total - 1;
+        const int t = (int)div_ll(slot, p.N);
+        const long long i = slot - (long long)t * p.N;
+        const bool uniform = __all_sync(full, t == __shfl_sync(full, t, 0));
+        float sc = 0.0f, acc = 0.0f, fa = 1.0f, ptx[2] = {0.0f, 0.0f};
+        f3 P = mk(0, 0, 0), n = mk(0, 0, 1), kr = mk(0, 0, 1);
+        int hit = -1, m = 0, am = -1;
+        if (in) {
+            const f3 o = mk(p.tx_pos[3 * t], p.tx_pos[3 * t + 1], p.tx_pos[3 * t + 2]);
+            const f3 d = p.dirs ? xyz(__ldg(p.dirs + i)) : fib_dir(p.N, i);
+            float th;
+            hit = closest_hit<false, LY>(p.s, nullptr, 0, o, d, -1, th, cnt);
+            if (hit >= 0) {
+                m = __ldg(p.s.mat + hit);
+                sc = fmaxf(__ldg(p.scat + m), 0.0f);   // S <= 0: no scattering
+                n = xyz(__ldg(p.s.planes + hit));
+                if (dot(d, n) > 0.0f) n = n * -1.0f;   // the side the ray came from
+                P = o + d * th;
+                am = p.alpha ? __ldg(p.alpha + m) : -1;
+                if (am >= 0) {
+                    const float dn = dot(d, n);                 // < 0: n faces the incoming ray
+                    kr = d - n * (2.0f * dn);
+                    fa = directive_norm(am, -dn) / RT_PI_F;     // pi / F_alpha replaces 1/pi in w0
+                }
+                const Rot<float> Rt = rot_ypr(p.tx_ypr[3 * t], p.tx_ypr[3 * t + 1], p.tx_ypr[3 * t + 2]);
+                for (int q = 0; q < p.txa.n_ports; q++) {
+                    const V3<float> f = antenna_vec<float>(p.txa.kind, p.txa.slant[q], Rt, V3<float>{d.x, d.y, d.z});
+                    ptx[q] = f.x * f.x + f.y * f.y + f.z * f.z;
+                }
+            }
+        }
+        if (!__any_sync(full, sc > 0.0f)) continue;
+        const int rb = p.rx_off ? p.rx_off[t] : 0, nr = (p.rx_off ? p.rx_off[t + 1] : p.n_rx) - rb;
+        const int nr_max = __reduce_max_sync(full, (unsigned)nr);
+        for (int k = 0; k < nr_max; k++) {
+            float w = 0.0f, prx[2] = {0.0f, 0.0f};
+            const int r = rb + k;
+            if (sc > 0.0f && k < nr) {
+                const f3 rx = mk(p.rx_pos[3 * r], p.rx_pos[3 * r + 1], p.rx_pos[3 * r + 2]);
+                const f3 v = rx - P;
+                const float dist = sqrtf(dot(v, v));
+                const float cs = dot(v, n) / dist;
+                const f3 ks = v * (1.0f / dist);
+                if (cs > 0.0f && !any_hit<false, LY>(p.s, nullptr, 0, P, ks, dist - p.s.tmin, hit, -1, cnt)) {
+                    const float pat = am < 0 ? cs : powf(0.5f * (1.0f + dot(kr, ks)), (float)am) / fa;
+                    w = (VJP ? 1.0f : sc * sc) * pat * p.w0 / (dist * dist);
+                    const Rot<float> Rr = rot_ypr(p.rx_ypr[3 * r], p.rx_ypr[3 * r + 1], p.rx_ypr[3 * r + 2]);
+                    for (int pp = 0; pp < p.rxa.n_ports; pp++) {
+                        const V3<float> f = antenna_vec<float>(p.rxa.kind, p.rxa.slant[pp], Rr, V3<float>{-ks.x, -ks.y, -ks.z});
+                        prx[pp] = f.x * f.x + f.y * f.y + f.z * f.z;
+                    }
+                }
+            }
+            const long long pair = p.rx_off ? (long long)r : (long long)t * p.n_rx + r;
+            if (VJP) {   // w is g / S^2 here
+                if (w != 0.0f)
+                    for (int pp = 0; pp < p.rxa.n_ports; pp++)
+                        for (int q = 0; q < p.txa.n_ports; q++)
+                            acc += __ldg(p.up + (pair * p.rxa.n_ports + pp) * p.txa.n_ports + q) * w * prx[pp] * ptx[q];
+                continue;
+            }
+            for (int pp = 0; pp < p.rxa.n_ports; pp++)
+                for (int q = 0; q < p.txa.n_ports; q++) {
+                    float c = w * prx[pp] * ptx[q];
+                    if (uniform)
+                        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(full, c, o);
+                    if (c != 0.0f && (!uniform || lane == 0))
+                        atomicAdd(p.gain + (pair * p.rxa.n_ports + pp) * p.txa.n_ports + q, c);
+                }
+        }
+        if (VJP && acc != 0.0f) atomicAdd((p.grad_smem ? sgrad : p.grad) + m, 2.0f * sc * acc);
     }
     if (VJP && p.grad_smem) {
         __syncthreads();
@@ -345,39 +444,37 @@ int scattering_impl(rt_ctx* ctx, int64_t N, float* gain, const float* up, float*
     // of six sites: 16 units 1.41 ms, 24 1.32, 32 1.35, 48 1.44: first hits against
     // the last wave's gap), to 32 rays and 4 receivers for one wave (2 x 1464 rays
     // x 127 receivers: 0.10 ms; one thread per ray and 64 receivers took 1.22 ms).
-    // Below 16 receivers a unit is a warp's 32 rays (1e5 rays x 1 receiver: 51 us,
-    // blocks of four warps 62).
     int nr_max = ctx->n_rx;
     if (ctx->rx_sets) {
         nr_max = 0;
         for (int t = 0; t < ctx->n_tx; t++) nr_max = std::max(nr_max, ctx->rx_off[t + 1] - ctx->rx_off[t]);
     }
-    const bool few = nr_max < 16;
-    const long long sms = ctx->num_sms, wave = (few ? 28 : 7) * sms;
+    const long long sms = ctx->num_sms, wave = 7 * sms;
     auto n_units = [&](int rays, long long chunks) { return (long long)ctx->n_tx * ((N + rays - 1) / rays) * chunks; };
     auto chunks_for = [&](int rays, long long units, int receivers) {
         return std::max<long long>(1, std::min<long long>(nr_max / receivers, (units + n_units(rays, 1) - 1) / n_units(rays, 1)));
     };
-    p.rays = few ? 32 : SC_RAYS;
-    if (!few && n_units(p.rays, std::max(1, nr_max / 32)) < 24 * sms) p.rays = 128;
+    // a thread a ray (k_scatter_few): for one receiver, and up to eight while units
+    // of 128 rays would make one to four waves, whose last one is partly empty
+    // (3e5 rays x 2 receivers: 82 us, k_scatter 93; x 8: 143 both; but 1e5 x 2: 72
+    // and 68, 1e6 x 2: 153 and 152, and 1e5 x 8: 107 and 87)
+    const long long coarse = n_units(128, 1);
+    const bool few = nr_max == 1 || (nr_max <= 8 && coarse > wave && coarse < 4 * wave);
+    p.rays = SC_RAYS;
+    if (n_units(p.rays, std::max(1, nr_max / 32)) < 24 * sms) p.rays = 128;
     p.n_chunks = (int)chunks_for(p.rays, 24 * sms, 32);
     if (n_units(p.rays, p.n_chunks) < wave) p.n_chunks = (int)chunks_for(p.rays, wave, 4);
     while (p.rays > 32 && n_units(p.rays, p.n_chunks) < wave) p.rays /= 2;
-    const unsigned blocks = (unsigned)std::min<long long>(n_units(p.rays, p.n_chunks), 1ll << 30);
-    const int threads = few ? 32 : 128;
+    const long long units = few ? std::min<long long>(((long long)ctx->n_tx * N + 127) / 128, 16 * sms)
+                                : std::min<long long>(n_units(p.rays, p.n_chunks), 1ll << 30);
     const size_t smem = p.grad_smem ? sizeof(float) * ctx->n_mat : 0;
     const bool wide = wide_layout(ctx);
-    if (vjp) {
-        prof_begin(ctx, "k_scatter_vjp");
-        auto kern = few ? (wide ? k_scatter<true, 8, 1> : k_scatter<true, 2, 1>)
-                        : (wide ? k_scatter<true, 8, 4> : k_scatter<true, 2, 4>);
-        kern<<<blocks, threads, smem, ctx->stream>>>(p);
-    } else {
-        prof_begin(ctx, "k_scatter");
-        auto kern = few ? (wide ? k_scatter<false, 8, 1> : k_scatter<false, 2, 1>)
-                        : (wide ? k_scatter<false, 8, 4> : k_scatter<false, 2, 4>);
-        kern<<<blocks, threads, 0, ctx->stream>>>(p);
-    }
+    auto kern = few ? (vjp ? (wide ? k_scatter_few<true, 8> : k_scatter_few<true, 2>)
+                           : (wide ? k_scatter_few<false, 8> : k_scatter_few<false, 2>))
+                    : (vjp ? (wide ? k_scatter<true, 8> : k_scatter<true, 2>)
+                           : (wide ? k_scatter<false, 8> : k_scatter<false, 2>));
+    prof_begin(ctx, vjp ? "k_scatter_vjp" : "k_scatter");
+    kern<<<(unsigned)units, 32 * SC_WARPS, smem, ctx->stream>>>(p);
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
     return RT_OK;

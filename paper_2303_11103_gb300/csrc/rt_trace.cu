@@ -88,13 +88,6 @@ __device__ __forceinline__ void stage_nodes(const TraceCommon& c, float4* sm) {
     __syncthreads();
 }
 
-// a / b for 0 <= a, 0 < b: in 32 bits where both fit, about a fifth of the
-// 64-bit division's instructions.
-__device__ __forceinline__ long long div_ll(long long a, long long b) {
-    if (((a | b) >> 32) == 0) return (unsigned)a / (unsigned)b;
-    return a / b;
-}
-
 // Warp-level ray fetch: when all lanes are dead, the next rays of the warp's
 // chunk. Lanes whose rays ended early wait for the others: the rays of a refill
 // start side by side and mostly hit the same surfaces, which a ray of another

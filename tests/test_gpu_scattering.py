@@ -199,3 +199,61 @@ def test_scattering_unit_edges(N, n_rx, n_tx):
             assert np.all(np.abs(got - og) <= tol), (t, np.abs(got - og).max(), og.max())
     finally:
         tr.close()
+
+
+@pytest.mark.parametrize("n_rx", [1, 9])
+def test_one_ray_exactly(n_rx):
+    """The single lattice ray (along +x) meets the box's wall; receivers that see it, against the oracle at
+    the tolerance of a well-conditioned value (one receiver: a thread a ray; nine: packed hits)."""
+    tr = rt.Tracer(0, FC)
+    try:
+        sc = S.tiny_scene()
+        tx = S.Devices(np.array([[-60.0, 1.0, 12.0]], np.float32), np.zeros((1, 3), np.float32), S.V_ISO)
+        rng = np.random.default_rng(5)
+        pos = np.stack([rng.uniform(-90.0, -20.0, n_rx), rng.uniform(-60.0, 60.0, n_rx), rng.uniform(1.0, 20.0, n_rx)], 1)
+        rx = S.Devices(pos.astype(np.float32), np.zeros((n_rx, 3), np.float32), S.V_ISO)
+        setup(tr, sc, tx, rx)
+        S_m = np.array([0.6], np.float32)
+        tr.set_scattering(S_m)
+        g = tr.scattering_gain(1).cpu().numpy()
+        og = SC.scattering_gain(O.make_scene(sc), sc.mat_id, S_m.astype(np.float64), FC, tx, rx, 1)
+        assert (og > 0.0).all()
+        assert np.all(np.abs(g - og) <= 2e-3 * og), (g, og)
+    finally:
+        tr.close()
+
+
+@pytest.mark.parametrize("width", [2, 8])
+@pytest.mark.parametrize("n_tx,N,n_rx,alpha", [(1, 3001, 1, -1),      # one receiver
+                                               (3, 33, 1, 4),         # warps over several transmitters
+                                               (2, 70001, 8, -1),     # units of 128 rays in a wave and a bit
+                                               (3, 50021, 5, 4)])
+def test_few_receivers(n_tx, N, n_rx, alpha, width):
+    """A thread a ray against packed hits: the same receivers alone and among
+    40 give the same gains and coefficient gradients, up to the order of
+    summation (fewer than 5000 partial sums a side, 2^-24 each)."""
+    tol = 2 * 5000 * 2.0 ** -24
+    sc = S.city_scene(n_side=6, size=150.0, seed=2)
+    rng = np.random.default_rng(N)
+    tx = np.concatenate([rng.uniform(-60.0, 60.0, (n_tx, 2)), np.full((n_tx, 1), 65.0)], 1).astype(np.float32)
+    rx = np.concatenate([rng.uniform(-74.0, 74.0, (40, 2)), rng.uniform(1.0, 70.0, (40, 1))], 1).astype(np.float32)
+    out = []
+    for n in (n_rx, 40):
+        tr = rt.Tracer(0, FC)
+        try:
+            tr.set_bvh_width(width)
+            tr.load_scene(sc)
+            tr.set_tx(tx, np.full((n_tx, 3), 0.1, np.float32), S.TR38901_VH)
+            tr.set_rx(rx[:n], np.zeros((n, 3), np.float32), S.V_ISO)
+            tr.set_scattering([0.3, 0.0, 0.6])
+            tr.set_scattering_pattern([alpha] * 3)
+            up = np.zeros((n_tx, n, 1, 2), np.float32)
+            up[:, :n_rx] = 1.0 + np.arange(n_rx)[None, :, None, None]
+            g = tr.scattering_gain(N).cpu().numpy().reshape(n_tx, n, 2)[:, :n_rx]
+            out.append((g, tr.scattering_gain_vjp(N, up.reshape(-1, 1, 2)).cpu().numpy()))
+        finally:
+            tr.close()
+    (ga, va), (gb, vb) = out
+    assert (gb > 0.0).any() and vb.max() > 0.0
+    assert np.all(np.abs(ga - gb) <= tol * gb + 1e-30)
+    assert np.all(np.abs(va - vb) <= tol * np.abs(vb) + 1e-30)
