@@ -335,12 +335,11 @@ __device__ __forceinline__ void flush_counts(TravCount& c, unsigned long long* c
 // The hierarchy is checked at build time to be a tree whose children have
 // larger indices than their parent (level order), with depth below
 // RT_STACK, so the loop visits each node at most once and the stack cannot
-// overflow. C: count node / triangle records and queries in cnt. TO: hits
-// before t_out's value on entry, and with `any` set the first one found.
-template <bool C, bool V8, bool TO = false>
+// overflow. C: count node / triangle records and queries in cnt.
+template <bool C, bool V8>
 __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm, int n_sm, f3 o, f3 d,
-                                             int exclude, float& t_out, TravCount& cnt, bool any = false) {
-    if (!TO) t_out = __int_as_float(0x7f800000);
+                                             int exclude, float& t_out, TravCount& cnt) {
+    t_out = __int_as_float(0x7f800000);
     if (C) cnt.queries++;
     if (s.n_tris == 0) return -1;
     f3 inv = safe_inv(d);
@@ -348,7 +347,7 @@ __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm
     int stack[RT_STACK];
     int sp = 0;
     int node = 0;
-    float tb = t_out;
+    float tb = __int_as_float(0x7f800000);
     int best = -1;
     const float tmin = s.tmin;
     // large triangles first: a hit there also bounds the traversal below
@@ -417,9 +416,8 @@ __device__ __forceinline__ int closest_hit_b(const DevScene& s, const float4* sm
             if (sp == 0) break;
             node = stack[--sp];
         }
-        if (TO && any && best >= 0) return best;
     }
-    if (!(TO && any)) t_out = tb;
+    t_out = tb;
     return best;
 }
 

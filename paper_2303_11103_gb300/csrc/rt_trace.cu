@@ -644,17 +644,22 @@ static TraceCommon make_common(rt_ctx* ctx, int64_t N, int64_t first, int64_t co
 }
 
 // Whether a trace takes its rays as beams: on the binary layout, with no
-// traversal counts asked for, in the direction-coherent order, and from
-// `density` rays per transmitter and triangle on: PK_DENSITY, twice that for the
-// orientation gradient, whose rays carry twice the registers. Wider beams meet
-// more triangles than a ray's own traversal does. Beams against single rays (us):
-// 4802 triangles, path trace of 32 transmitters, depth 3, 2e4 rays each 456 / 240,
-// 6e4 451 / 433, 2e5 775 / 1024; map of 8 x 1e5 250 / 223, 4 x 1e6 702 / 939;
-// gradient of 2 x 3e5 278 / 240; 770 triangles: path trace 2e4 207 / 237, 6e4
-// 317 / 533, gradient of 4 x 1.5e4 208 / 146, 2 x 3e5 208 / 344.
+// traversal counts asked for, in the direction-coherent order, in scenes of
+// PK_TRIS triangles on (one box on its ground, 14 triangles: 1 to 1.3 times the
+// time of single rays at any ray count; 50 triangles 0.3 to 0.98), and from
+// `density` rays per transmitter and triangle on: wider beams meet more triangles
+// than a ray's own traversal does. Time as beams over time ray by ray, geometric
+// means over 21 cities of 302 to 6914 triangles, at 40, 60, 80, 120 rays a
+// triangle: map of one transmitter, depth 1 0.88 0.86 0.85 0.80, depth 3 0.94 0.89
+// 0.88 0.82, depth 5 0.97 0.95 0.97 0.90, of four 0.82 .. 0.74, 0.94 .. 0.77, 1.01
+// 0.92 0.89 0.82 (single sites up to 1.3 at 40, 1.2 at 120); path trace, depth 3,
+// one 0.96 .. 0.85, four 0.94 .. 0.80; orientation gradient, depth 3, one 0.98 0.89
+// 0.88 0.80, depth 5 1.05 0.98 0.98 0.88, of four 0.99 0.90 0.90 0.83 (sites up to
+// 1.4 below 80, where the gain is small: twice the density there).
 constexpr long long PK_DENSITY = 40;
+constexpr int PK_TRIS = 32;
 static bool use_beams(const rt_ctx* ctx, const TraceCommon& c, long long density = PK_DENSITY) {
-    return !wide_layout(ctx) && !ctx->count_work && c.perm && ctx->n_tris > 0 && c.N >= density * ctx->n_tris;
+    return !wide_layout(ctx) && !ctx->count_work && c.perm && ctx->n_tris >= PK_TRIS && c.N >= density * ctx->n_tris;
 }
 
 // Shoot and bounce: appends every hit's candidate key with its position
