@@ -84,7 +84,10 @@ int rt_set_frequency(rt_ctx* ctx, double fc);
  * verts [n_tris*9] float32 (v0, v1, v2 of each triangle), mat_id [n_tris]
  * int32 in [0, n_mat), mat_params [n_mat*2] float32 (eps_r, sigma).
  * Builds the LBVH on the GPU. Surfaces are two-sided. n_tris may be 0
- * (every ray misses). Errors: RT_ERR_INVALID_ARG, RT_ERR_OOM, RT_ERR_CUDA.
+ * (every ray misses). For the binary layout it also lays out the boxes that
+ * neighbouring rays traverse together (290 bytes a triangle beside about 750 of
+ * records and nodes; 35 us of the 320 a load of 4802 triangles takes). Errors:
+ * RT_ERR_INVALID_ARG, RT_ERR_OOM, RT_ERR_CUDA.
  */
 int rt_load_scene(rt_ctx* ctx, const float* verts, int64_t n_tris, const int32_t* mat_id,
                   const float* mat_params, int32_t n_mat);
@@ -108,7 +111,8 @@ int rt_set_bvh_builder(rt_ctx* ctx, int32_t builder);
  * reads each child's near and far planes by its direction octant, visiting
  * children near to far. Both give the same intersections. On the
  * 4802-triangle city the binary layout is the faster one (fewer box tests
- * per query). Takes effect at the next rt_load_scene. Errors:
+ * per query). Takes effect at the next rt_load_scene; a scene loaded at width
+ * 8 is traversed ray by ray after a change to 2 until then. Errors:
  * RT_ERR_INVALID_ARG for another width.
  */
 int rt_set_bvh_width(rt_ctx* ctx, int32_t width);

@@ -89,7 +89,7 @@ DevScene dev_scene(rt_ctx* ctx) {
     s.n_nodes = ctx->n_nodes;
     s.n_mat = ctx->n_mat;
     s.tmin = ctx->tmin;
-    s.pk = bp<float4>(ctx->pk);
+    s.pk = ctx->pk_ok ? bp<float4>(ctx->pk) : nullptr;
     s.pk_rho = 0.5f * ctx->extent / std::sqrt((float)std::max((ctx->n_bvh + 31) / 32, 1));
     return s;
 }

@@ -992,10 +992,47 @@ __global__ void __launch_bounds__(1024) k_pk_boxes(const float4* __restrict__ tr
     if (lane == 0) put(b2 + blockIdx.x, b, 0);
 }
 
+// The boxes that beams traverse (rt_packet.cuh), from the leaf records of the
+// scene's bounds `bounds` (lo, hi). The caller reads the radix sort's status.
+static int build_pk(rt_ctx* ctx, const float (&bounds)[6], float ext, float scale) {
+    cudaStream_t st = ctx->stream;
+    const int n = ctx->n_bvh, n_big = ctx->n_big, B = 256;
+    const int groups = (n + 31) / 32, sets = (groups + 31) / 32;
+    RT_TRY(buf_reserve(ctx->pk, 32 * (1 + 8 * 32 * ((size_t)groups + sets + (sets + 31) / 32 + (n_big + 31) / 32))));
+    // flat scenes: leaves along a Hilbert curve over the two long axes, whose runs
+    // of 32 are more compact than the Morton order's (city: 129 m of width and
+    // depth against 159; 64-transmitter map 91.8 -> 80.7 ms, city map 190 -> 163 us)
+    const uint32_t* order = nullptr;
+    const float* lo = bounds;
+    float side[3];
+    for (int k = 0; k < 3; k++) side[k] = bounds[3 + k] - lo[k];
+    const int thin = side[2] <= side[0] && side[2] <= side[1] ? 2 : side[1] <= side[0] ? 1 : 0;
+    const int ax = thin == 0 ? 1 : 0, ay = thin == 2 ? 1 : 2;
+    if (n > 32 && 4.0f * side[thin] <= std::min(side[ax], side[ay])) {
+        RT_TRY(buf_reserve(ctx->pk_order, (2 * sizeof(uint64_t) + 2 * sizeof(uint32_t)) * (size_t)n));
+        uint64_t *k0 = bp<uint64_t>(ctx->pk_order), *k1 = k0 + n;
+        uint32_t *v0 = reinterpret_cast<uint32_t*>(k1 + n), *v1 = v0 + n;
+        prof_begin(ctx, "k_pk_keys");
+        k_pk_keys<<<(n + B - 1) / B, B, 0, st>>>(bp<float4>(ctx->tris), n, ax, ay, lo[ax], lo[ay], ext / 65536.0f, k0, v0);
+        prof_end(ctx);
+        RT_TRY(cudaGetLastError());
+        RT_TRY(radix_sort64(ctx, k0, k1, v0, v1, n, 32));
+        order = v0;
+    }
+    prof_begin(ctx, "k_pk_boxes");
+    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), order, n, n_big, 4e-6f * scale, groups, sets,
+                                          bp<float4>(ctx->pk));
+    prof_end(ctx);
+    RT_TRY(cudaGetLastError());
+    ctx->pk_ok = true;
+    return RT_OK;
+}
+
 int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     const int T = (int)n_tris;
     cudaStream_t st = ctx->stream;
     ctx->n_tris = T;
+    ctx->pk_ok = false;
     if (T == 0) {
         ctx->n_nodes = 0;
         ctx->n_bvh = ctx->n_big = 0;
@@ -1257,35 +1294,15 @@ int bvh_build(rt_ctx* ctx, const float* verts, int64_t n_tris) {
     k_leaf_tris<<<gT, B, 0, st>>>(T, leaf_tri, bp<float4>(ctx->tris_o), bp<float4>(ctx->tris));
     prof_end(ctx);
     RT_TRY(cudaGetLastError());
-    const int groups = (n + 31) / 32, sets = (groups + 31) / 32;
-    RT_TRY(buf_reserve(ctx->pk, 32 * (1 + 8 * 32 * ((size_t)groups + sets + (sets + 31) / 32 + (n_big + 31) / 32))));
-    // flat scenes: leaves along a Hilbert curve over the two long axes, whose runs
-    // of 32 are more compact than the Morton order's (city: 129 m of width and
-    // depth against 159; 64-transmitter map 91.8 -> 80.7 ms, city map 190 -> 163 us)
-    const uint32_t* order = nullptr;
-    float lo[3], side[3];
-    for (int k = 0; k < 3; k++) {
-        lo[k] = host_unord(hi[k]);
-        side[k] = host_unord(hi[3 + k]) - lo[k];
+    // the 8-wide layout traverses ray by ray: no boxes for beams (a width of 2 set
+    // without another load goes ray by ray too). 4802 triangles, width 8: 462 us
+    // a load without, 491 with; 120002 triangles: 35 MB less.
+    if (ctx->bvh_width != 8 || n < 2) {
+        float bounds[6];
+        for (int k = 0; k < 6; k++) bounds[k] = host_unord(hi[k]);
+        const int e = build_pk(ctx, bounds, ext, scale);
+        if (e) return e;
     }
-    const int thin = side[2] <= side[0] && side[2] <= side[1] ? 2 : side[1] <= side[0] ? 1 : 0;
-    const int ax = thin == 0 ? 1 : 0, ay = thin == 2 ? 1 : 2;
-    if (n > 32 && 4.0f * side[thin] <= std::min(side[ax], side[ay])) {
-        RT_TRY(buf_reserve(ctx->pk_order, (2 * sizeof(uint64_t) + 2 * sizeof(uint32_t)) * (size_t)n));
-        uint64_t *k0 = bp<uint64_t>(ctx->pk_order), *k1 = k0 + n;
-        uint32_t *v0 = reinterpret_cast<uint32_t*>(k1 + n), *v1 = v0 + n;
-        prof_begin(ctx, "k_pk_keys");
-        k_pk_keys<<<(n + B - 1) / B, B, 0, st>>>(bp<float4>(ctx->tris), n, ax, ay, lo[ax], lo[ay], ext / 65536.0f, k0, v0);
-        prof_end(ctx);
-        RT_TRY(cudaGetLastError());
-        RT_TRY(radix_sort64(ctx, k0, k1, v0, v1, n, 32));
-        order = v0;
-    }
-    prof_begin(ctx, "k_pk_boxes");
-    k_pk_boxes<<<sets + 1, 1024, 0, st>>>(bp<float4>(ctx->tris), order, n, (int)n_big, 4e-6f * scale, groups, sets,
-                                          bp<float4>(ctx->pk));
-    prof_end(ctx);
-    RT_TRY(cudaGetLastError());
     ctx->n_wnodes = 0;
     if (n >= 2) {
         RT_TRY(cudaMemcpyAsync(ctx->host_rb, info + 13, sizeof(hd), cudaMemcpyDeviceToHost, st));

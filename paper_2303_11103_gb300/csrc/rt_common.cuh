@@ -73,7 +73,7 @@ struct DevScene {
     const float2* __restrict__ mats;    // [M] eps_r, sigma
     int n_tris, n_nodes, n_mat, n_big;
     float tmin;                         // self-intersection offset (metres)
-    const float4* __restrict__ pk;      // boxes for traversal by beams (rt_packet.cuh)
+    const float4* __restrict__ pk;      // boxes for traversal by beams (rt_packet.cuh), or null
     float pk_rho;                       // spread of a beam's origins (metres)
 };
 

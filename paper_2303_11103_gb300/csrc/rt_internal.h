@@ -46,7 +46,8 @@ struct rt_ctx {
     DevBuf wnodes;        // 8-wide layout [n_wnodes * RT_WN_F4] (when bvh_width == 8)
     int n_wnodes = 0;
     DevBuf planes64;   // [T*3] double2: FP64 unit normal and first vertex per triangle (original order)
-    DevBuf pk;                 // boxes for traversal by beams (rt_packet.cuh)
+    DevBuf pk;                 // boxes for traversal by beams (rt_packet.cuh), of this scene when pk_ok
+    bool pk_ok = false;        // (a scene loaded for the 8-wide layout has none)
     DevBuf pk_order;           // build scratch: order of their leaves
 
     // devices

@@ -209,7 +209,8 @@ __device__ __forceinline__ void beam_trace(const DevScene& s, bool mine, bool an
 // Any occluder (any_hit) of the segments from o to e, d = (e - o) / |e - o|, for
 // the lanes of `need`, called by all 32: those that start and end near the
 // first one's ends as a beam, the others one by one. found: the occluder
-// (index in s.tris), or RT_NO_REF. Layout 8: all one by one, no occluder named.
+// (index in s.tris), or RT_NO_REF. Without boxes for beams all one by one; layout
+// 8: no occluder named either.
 template <int LY>
 __device__ __forceinline__ bool warp_segments(const DevScene& s, bool need, f3 o, f3 e, f3 d, float tmax, int ex0, int ex1,
                                               int& found) {
@@ -229,7 +230,7 @@ __device__ __forceinline__ bool warp_segments(const DevScene& s, bool need, f3 o
     const bool in = need && (lane == lead || (fmax3(fabsf(ox), fabsf(oy), fabsf(oz)) <= rho &&
                                               fmax3(fabsf(ex), fabsf(ey), fabsf(ez)) <= rho));
     const unsigned m = __ballot_sync(full, in);
-    const bool beam = __popc(m) >= PK_MIN;
+    const bool beam = s.pk && __popc(m) >= PK_MIN;
     if (beam) {
         Beam b;
         b.x = seg_axis(in, o.x, e.x);

@@ -659,7 +659,8 @@ static TraceCommon make_common(rt_ctx* ctx, int64_t N, int64_t first, int64_t co
 constexpr long long PK_DENSITY = 40;
 constexpr int PK_TRIS = 32;
 static bool use_beams(const rt_ctx* ctx, const TraceCommon& c, long long density = PK_DENSITY) {
-    return !wide_layout(ctx) && !ctx->count_work && c.perm && ctx->n_tris >= PK_TRIS && c.N >= density * ctx->n_tris;
+    return !wide_layout(ctx) && ctx->pk_ok && !ctx->count_work && c.perm && ctx->n_tris >= PK_TRIS &&
+           c.N >= density * ctx->n_tris;
 }
 
 // Shoot and bounce: appends every hit's candidate key with its position

@@ -129,3 +129,31 @@ def test_handed_out_validation_units(n_rx, sets):
     assert len(a["depth"]) > 1000
     for k in a:
         assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("n", [1, 2, 3000])
+def test_width_changed_without_a_load(n):
+    """A scene loaded for the 8-wide layout has no boxes for beams: set to the
+    binary layout it is traversed ray by ray, with the same hits, map counts and
+    diffracted paths (one triangle: no wide nodes either, so it has the boxes)."""
+    sc = _soup(n, 1, 6) if n < 100 else _city(6)
+    rays = 40 * sc.n_tris + 100
+    grid = dict(x0=-60.0, y0=-60.0, cell=6.0, nx=20, ny=20, h=1.5)
+    out = []
+    for first in (2, 8):
+        tr = rt.Tracer(0, FC)
+        try:
+            tr.set_bvh_width(first)
+            tr.load_scene(sc)
+            tr.set_bvh_width(2)
+            tr.set_tx(np.array([[3.0, -4.0, 40.0]], np.float32), np.zeros((1, 3), np.float32), S.V_ISO)
+            tr.set_rx(np.array([[10.0, 5.0, 1.5]] * 40, np.float32), np.zeros((40, 3), np.float32), S.V_ISO)
+            tr.compute_paths(2, rays, record_rays=True)
+            hits = tr.ray_hits().cpu().numpy()
+            count = tr.coverage_map(grid, 2, rays)[1].cpu().numpy()
+            tr.compute_diffraction()
+            out.append((hits, count, tr.diffraction()["wedge"].cpu().numpy()))
+        finally:
+            tr.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
