@@ -38,7 +38,7 @@
 // where the rays are dense; a limit on a beam's triangle tests, 16 to 64, cost
 // 2 to 10 %.)
 constexpr float PK_DIR = 0.2f;
-constexpr int PK_MIN = 12, PK_FEW = 16, PK_BEAMS = 3;
+constexpr int PK_MIN = 12, PK_FEW = 16, PK_BEAMS = 4;
 
 __device__ __forceinline__ float warp_min(float x) {
     float r;
@@ -315,7 +315,7 @@ __device__ __forceinline__ void warp_trace(const DevScene& s, bool need, bool an
     if (s.n_tris == 0) return;
     // each ray's beam: the first ray of those not yet in one and what lies near it
     int mine = -1, beams = 0;
-    while (todo && beams <= PK_BEAMS) {
+    while (todo && beams < PK_BEAMS) {
         const int lead = __ffs(todo) - 1;
         const float dx = d.x - __shfl_sync(full, d.x, lead), dy = d.y - __shfl_sync(full, d.y, lead),
                     dz = d.z - __shfl_sync(full, d.z, lead);
