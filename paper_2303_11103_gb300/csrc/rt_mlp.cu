@@ -317,6 +317,8 @@ constexpr uint32_t WG_STAGE = 2 * WG_CHUNK + WG_ROWS * WG_N * 2;
 struct WgradArgs {
     int W, K0, L, B;
     int64_t cap;   // rows between consecutive layers of dZ (and of H)
+    int layer;     // the only layer of this launch, or -1: all
+    int64_t z0;    // first row of its dZ
     float* g;      // gradient vector
     unsigned* err;
 };
@@ -345,7 +347,9 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ CUtens
     // layer, 128-output tile and 32-input tile of this CTA
     const int mt = (a.W + 127) / 128, nt0 = (a.K0 + WG_N - 1) / WG_N, nt1 = a.W / WG_N;
     int l, t = blockIdx.x;
-    if (t < mt * nt0) {
+    if (a.layer >= 0) {
+        l = a.layer;
+    } else if (t < mt * nt0) {
         l = 0;
     } else {
         t -= mt * nt0;
@@ -378,7 +382,7 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ CUtens
     // the layer's place in the gradient vector (W then b of every layer)
     float* out = a.g + (l == 0 ? 0 : (int64_t)a.W * a.K0 + a.W + (int64_t)(l - 1) * (a.W * a.W + a.W));
     if (warp == 0 && lane == 0) {
-        const int zr = (int)(l * a.cap), hr = l == 0 ? 0 : (int)((l - 1) * a.cap);
+        const int zr = (int)(a.layer >= 0 ? a.z0 : l * a.cap), hr = l == 0 ? 0 : (int)((l - 1) * a.cap);
         const CUtensorMap* mh = l == 0 ? &th0 : &th;
         int issued = 0;
         for (int kb = 0; kb < nkb; kb++, issued++) {
@@ -1295,6 +1299,7 @@ struct rt_mlp {
     DevBuf hpart;         // partial sums of the head's gradients (k_head_bwd)
     int64_t cap = 0;      // rows of the activation buffers
     int64_t tcap = 0;     // rows of the training buffers
+    int zl = 0;           // layers that dZ holds: L, or 2 in turn where memory has no room for all
     int step = 0;
     int in_dim(int l) const { return l == 0 ? 2 * F : W; }
     int out_dim(int l) const { return l == L ? 2 : W; }
@@ -1335,8 +1340,15 @@ static int mlp_reserve_train(rt_mlp* m, int64_t B) {
     if (m->cap <= m->tcap) return RT_OK;
     m->tcap = 0;
     MT(buf_reserve(m->dy, sizeof(float) * 2 * m->cap));
-    MT(buf_reserve(m->dZ, sizeof(__nv_bfloat16) * m->cap * m->W * m->L));
     MT(buf_reserve(m->hpart, sizeof(float) * (size_t)(m->cap / HB_ROWS + 1) * (2 * m->W + 2)));
+    const size_t layer = sizeof(__nv_bfloat16) * (size_t)m->cap * m->W;
+    m->zl = m->L;
+    cudaError_t e = buf_reserve(m->dZ, layer * m->L);
+    if (e == cudaErrorMemoryAllocation && m->L > 2) {
+        m->zl = 2;
+        e = buf_reserve(m->dZ, layer * 2);
+    }
+    MT(e);
     m->tcap = m->cap;
     return RT_OK;
 }
@@ -1568,23 +1580,8 @@ int rt_mlp_train_step(rt_mlp* m, const float* x, const float* target, int32_t B,
     int NS = 0;
     for (int n = 4; n >= 2 && !NS; n--)
         if (1024 + TrainLayout(m->F, W, L, n).bytes(n) <= 227 * 1024) NS = n;
-    if (K0 % 64 == 0 && NS) {
-        rc = launch_train_chain(m, x, target, B, loss, NS);
-        if (rc) return rc;
-    } else {
-        rc = mlp_forward(m, x, B);
-        if (rc) return rc;
-        k_loss<<<(B + 255) / 256, 256, 0, st>>>(bp<float>(m->y), target, x, B, m->db_scale, m->db_offset, m->lam,
-                                               bp<float>(m->dy), loss);
-        auto dz = [&](int l) { return bp<__nv_bfloat16>(m->dZ) + (size_t)l * m->cap * W; };
-        k_head_bwd<<<B / HB_ROWS, W / 2, 0, st>>>(m->hid(L), bp<float>(m->dy), W, m->wp(L), dz(L - 1),
-                                                  bp<float>(m->hpart));
-        MT(cudaGetLastError());
-        // dH_l = dZ_l W_l, then through the ReLU of layer l's input
-        for (int l = L - 1; l > 0; l--)
-            MT(gemm_bf16(st, dz(l), m->wtb(l), B, W, W, nullptr, 0, 1, dz(l - 1), W, err, m->hid(l)));
-    }
-    // dW_l = dZ_l^T H_l and the bias gradients of all hidden layers
+    const bool all_dz = m->zl == L;
+    // dW_l = dZ_l^T H_l and the bias gradients of all hidden layers, or of one
     WgradArgs wa;
     wa.W = W;
     wa.K0 = K0;
@@ -1594,15 +1591,41 @@ int rt_mlp_train_step(rt_mlp* m, const float* x, const float* target, int32_t B,
     wa.g = bp<float>(m->g);
     wa.err = err;
     alignas(64) CUtensorMap tz, th0, th;
-    if (!make_map(&tz, m->dZ.p, (uint64_t)L * m->cap, W, WG_ROWS) ||
+    if (!make_map(&tz, m->dZ.p, (uint64_t)m->zl * m->cap, W, WG_ROWS) ||
         !make_map(&th0, m->H0.p, m->cap, K0, WG_ROWS, WG_N) ||
         !make_map(&th, m->H.p, (uint64_t)L * m->cap, W, WG_ROWS, WG_N))
         return mlp_err(m, RT_ERR_CUDA, "tensor map of the training buffers");
     const size_t smem = 1024 + (size_t)WG_ST * WG_STAGE;
     MT(ensure_smem_attr((const void*)k_wgrad, smem));
-    const int tiles = (W + 127) / 128 * ((K0 + WG_N - 1) / WG_N + (L - 1) * (W / WG_N));
-    k_wgrad<<<(unsigned)tiles, 128, smem, st>>>(tz, th0, th, wa);
-    MT(cudaGetLastError());
+    const int mt = (W + 127) / 128, nt0 = (K0 + WG_N - 1) / WG_N, nt1 = W / WG_N;
+    auto wgrad = [&](int layer, int slot) -> cudaError_t {
+        wa.layer = layer;
+        wa.z0 = (int64_t)slot * m->cap;
+        const int tiles = mt * (layer < 0 ? nt0 + (L - 1) * nt1 : layer == 0 ? nt0 : nt1);
+        k_wgrad<<<(unsigned)tiles, 128, smem, st>>>(tz, th0, th, wa);
+        return cudaGetLastError();
+    };
+    if (K0 % 64 == 0 && NS && all_dz) {
+        rc = launch_train_chain(m, x, target, B, loss, NS);
+        if (rc) return rc;
+    } else {
+        rc = mlp_forward(m, x, B);
+        if (rc) return rc;
+        k_loss<<<(B + 255) / 256, 256, 0, st>>>(bp<float>(m->y), target, x, B, m->db_scale, m->db_offset, m->lam,
+                                               bp<float>(m->dy), loss);
+        // where a layer's gradient lies
+        auto slot = [&](int l) { return all_dz ? l : l & 1; };
+        auto dz = [&](int l) { return bp<__nv_bfloat16>(m->dZ) + (size_t)slot(l) * m->cap * W; };
+        k_head_bwd<<<B / HB_ROWS, W / 2, 0, st>>>(m->hid(L), bp<float>(m->dy), W, m->wp(L), dz(L - 1),
+                                                  bp<float>(m->hpart));
+        MT(cudaGetLastError());
+        // dH_l = dZ_l W_l, then through the ReLU of layer l's input
+        for (int l = L - 1; l >= 0; l--) {
+            if (!all_dz) MT(wgrad(l, slot(l)));   // before the layer below the next takes its place
+            if (l > 0) MT(gemm_bf16(st, dz(l), m->wtb(l), B, W, W, nullptr, 0, 1, dz(l - 1), W, err, m->hid(l)));
+        }
+    }
+    if (all_dz) MT(wgrad(-1, 0));
     m->step++;
     AdamArgs aa;
     aa.W = W;

@@ -192,3 +192,28 @@ def test_train_step_shapes(F, W, L, B, first):
 def test_train_step_chunks(F, W, L, B):
     """One fused step where warps share a chunk or two stored-only chunks follow each other."""
     test_train_step_shapes(F, W, L, B, 0)
+
+
+def test_train_step_where_memory_is_short():
+    """A batch whose gradients of all layers do not fit beside the activations: two layers' in turn, the same
+    gradients."""
+    F, W, L, B = 32, 256, 16, 1 << 21   # 17.2 GB of hidden outputs, as much of gradients
+    x = torch.rand((B, 6), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    t = torch.stack([(x[:, 0] < 0.5).float(), -140.0 + 70.0 * x[:, 1]], 1).contiguous()
+    out = []
+    torch.cuda.empty_cache()
+    for short in (True, False):
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - 24 * 10 ** 9, dtype=torch.uint8, device="cuda") if short else None
+        S = rt.Surrogate(np.zeros(6), np.ones(6), n_freq=F, width=W, n_hidden=L, seed=3)
+        try:
+            S.train_step(x, t, 0.0)
+            out.append(S.grads().cpu().numpy())
+            torch.cuda.synchronize()
+            assert S.status() == 0
+            assert not short or torch.cuda.mem_get_info()[0] > 2 * 10 ** 9   # all layers' would have left none
+        finally:
+            S.close()
+            del hog
+            torch.cuda.empty_cache()
+    assert np.abs(out[1]).max() > 0.0
+    assert np.array_equal(out[0], out[1])
