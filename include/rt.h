@@ -554,7 +554,8 @@ int rt_graph_launch(rt_ctx* ctx);
 int rt_autotune(rt_ctx* ctx, const rt_grid* g, int32_t max_depth, int64_t num_rays, float* gain,
                 uint32_t* hits, const char* cache_path);
 /* The launch configuration in use: block threads (128|256), rays per warp
- * refill (0 = automatic, else >= 32), BVH nodes staged in shared memory
+ * refill (0 = automatic: 32, or fewer, down to 4, for launches of too few
+ * rays to fill the GPU; else >= 32), BVH nodes staged in shared memory
  * (<= 3200, counted in 64-byte binary nodes; used by the 8-wide layout
  * only, the binary layout reads its octant copies through L1) (HOST out /
  * in). */

@@ -164,8 +164,8 @@ __device__ __forceinline__ bool tile_reached(const CellGrid& g, int tile, int ti
 // receiver tiles, a lane per receiver, so the wedge's record, its exterior
 // normal and the transmitter's side of Keller's law are computed once per run
 // and neighbouring lanes test nearby segments. The occluder that last blocked
-// tx -> D (and D -> rx) for this run is tried first (ref_hit: one box and one
-// triangle instead of a traversal); the candidates it does not block are
+// tx -> D (and D -> rx) for this run is tried first (ref_hit: one triangle
+// instead of a traversal); the candidates it does not block are
 // queued, so that the traversals run with all 32 lanes.
 //
 // The queued segments of a warp lie side by side (one wedge, neighbouring cells)

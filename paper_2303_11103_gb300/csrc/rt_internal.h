@@ -123,7 +123,7 @@ struct rt_ctx {
     int bvh_width = 2;              // traversal layout: 2 (binary nodes) or 8 (wide nodes)
     int dedup = RT_DEDUP_HASH;      // candidate duplicate removal: RT_DEDUP_HASH or RT_DEDUP_SORT
     int trace_block = 256;
-    int warp_chunk = 0;       // rays a warp takes per refill (0 = automatic: 32)
+    int warp_chunk = 0;       // rays a warp takes per refill (0 = automatic: 4 to 32, pick_chunk)
 
     // instrumentation: host count of kernel launches; optional CUDA-event
     // timing of every launch on the context's stream

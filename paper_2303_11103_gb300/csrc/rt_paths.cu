@@ -950,7 +950,8 @@ int compute_paths_impl(rt_ctx* ctx, int D, int64_t N, uint32_t flags, int64_t* o
             const int64_t units = nkeys * per_cand;
             const int64_t need = (units + 7) / 8;   // 8 warps per block
             const int64_t grid = std::max<int64_t>(std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * ctx->num_sms), 1);
-            // every warp gets about 64 units (n_uniq: distinct candidates, where known)
+            // every warp gets about 64 units (n_uniq: distinct candidates; the sort of
+            // RT_DEDUP_SORT leaves them on the device, so that mode always deals)
             if (!wide_layout(ctx) && !ctx->count_work && n_uniq * per_cand >= 64 * 8 * grid) {
                 kern = k_validate<false, 2, true>;
                 RT_TRY(ensure_smem_attr((const void*)kern, smem));
