@@ -4,6 +4,7 @@ by ray; the binary layout takes beams from 40 rays per triangle on, so the same
 scene on both gives both sides."""
 import numpy as np
 import pytest
+import torch
 
 from paper_2303_11103_gb300 import rt
 from paper_2303_11103_gb300 import scenes as S
@@ -157,3 +158,51 @@ def test_width_changed_without_a_load(n):
             tr.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("sets", [False, True])
+def test_validation_units_on_one_layout(sets):
+    """The binary layout against itself: the hash leaves the host the number of
+    candidates, so that the validation hands out its units, the sort does not,
+    so that they are dealt. The kernels that ran are read from a trace."""
+    sc = _city(8)
+    rng = np.random.default_rng(3)
+    n_tx, n_rx = 8, 2000
+    pos = np.concatenate([rng.uniform(-80.0, 80.0, (n_tx, 2)), rng.uniform(30.0, 60.0, (n_tx, 1))], 1).astype(np.float32)
+    cut = [0, 3000, 3000, 5001, 9000, 9001, 12000, 14000, 15990] if sets else None
+    n = cut[-1] if sets else n_rx
+    rx = np.concatenate([rng.uniform(-95.0, 95.0, (n, 2)), np.full((n, 1), 1.5)], 1).astype(np.float32)
+    out, ran = [], []
+
+    def trace():
+        return torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA])
+
+    with trace():   # the process's first trace may come back empty
+        torch.zeros(1, device="cuda").add_(1)
+        torch.cuda.synchronize()
+    for mode in (rt.DEDUP_HASH, rt.DEDUP_SORT):
+        tr = rt.Tracer(0, FC)
+        try:
+            tr.set_dedup(mode)
+            tr.load_scene(sc)
+            tr.set_tx(pos, np.zeros((n_tx, 3), np.float32), S.V_ISO)
+            tr.set_rx(rx, np.zeros((n, 3), np.float32), S.V_ISO, cut)
+            with trace() as prof:
+                tr.compute_paths(3, 200000)
+                torch.cuda.synchronize()
+            ran.append({e.name for e in prof.events() if "k_validate" in e.name})
+            out.append({k: v.cpu().numpy() for k, v in tr.paths().items()})
+            per_candidate = ((n if sets else n_tx * n_rx) // n_tx + 31) // 32
+            units = len(tr.candidates()[0]) * per_candidate
+        finally:
+            tr.close()
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert units >= 64 * 8 * 4 * sms   # the rule, at 4 blocks of 8 warps on an SM
+    a, b = out
+    assert len(a["depth"]) > 1000
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
+    if not any(ran):
+        pytest.skip("the profiler recorded no kernels: the paths agree, which kernel gave them is not shown")
+    handed = ["true>" in names.pop() for names in ran if len(names) == 1]   # k_validate's last parameter
+    assert handed == [True, False], ran
