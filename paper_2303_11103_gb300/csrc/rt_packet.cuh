@@ -272,6 +272,7 @@ __device__ __forceinline__ int single_ray(const DevScene& s, bool any, f3 o, f3 
             }
         }
     };
+#pragma unroll 1
     for (int k = 0; k < s.n_big; k++) test(s.big + 3 * k);
     const float4* onodes = octant_nodes(s, inv);
     const PairRay pr = pair_ray(inv, oi);
@@ -337,6 +338,8 @@ __device__ __forceinline__ void warp_trace(const DevScene& s, bool need, bool an
         else beam_trace(s, mine == n, any, o, d, ex, t, id);
     }
     rest |= todo;
-    if ((rest >> lane) & 1u) id = single_ray(s, any, o, d, ex, t);
-    __syncwarp();
+    if (rest) {   // for the warp: its set-up is not computed where all went as beams
+        if ((rest >> lane) & 1u) id = single_ray(s, any, o, d, ex, t);
+        __syncwarp();
+    }
 }
