@@ -482,8 +482,8 @@ ALU_PEAK_GOPS = 152 * 128 * 2.070
 K_COVERAGE_TRAFFIC = 21.33e6
 # L1/TEX throughput of the same launch (% of its peak, elapsed) and the
 # sector hit rate: the traversal's record reads are served by L1.
-K_COVERAGE_L1 = {"l1tex_throughput_pct": 31.9, "l1tex_sector_hit_pct": 88.1, "lts_throughput_pct": 3.5,
-                 "source": "profiles/k_coverage_city_1e6rays.md (ncu --set full, one launch)"}
+K_COVERAGE_L1 = {"l1tex_throughput_pct": 30.8, "l1tex_sector_hit_pct": 88.1, "lts_throughput_pct": 3.5,
+                 "source": "profiles/k_coverage_city_1e6rays.md (ncu, one launch)"}
 
 
 def traversal_probe(ctx, counts, n_tri=4):

@@ -176,7 +176,7 @@ __device__ __forceinline__ bool tile_reached(const CellGrid& g, int tile, int ti
 //
 // Bound by the candidates' own arithmetic and by the segments no kept
 // occluder answers. City map of 500 x 500 cells x 4800 wedges (1.2e9
-// candidates), mean of six sites: 4.1 ms; 73 to 87 ms with one thread per
+// candidates), mean of six sites: about 4.0 ms; 73 to 87 ms with one thread per
 // (receiver, wedge) in wedge order (7.6 of 32 lanes active, the wedge reloaded
 // and its sincos and transmitter side recomputed per candidate). On the way, at
 // one site: 12.8 ms a warp a wedge, 9.8 segments as beams, 6.3 tiles left out,
