@@ -536,7 +536,8 @@ int rt_freq_response_backward(rt_ctx* ctx, const float* a, const float* tau, con
  * replays). One graph per context; rt_graph_begin replaces the previous.
  * A replay is refused (RT_ERR_NOT_READY) once a later call has reallocated
  * a context buffer the graph uses (a larger scene or device set, another
- * ray count): capture again.
+ * ray count), or loaded a scene with other counts of triangles, nodes or
+ * materials or for the other node layout: capture again.
  */
 int rt_graph_begin(rt_ctx* ctx);
 int rt_graph_end(rt_ctx* ctx);

@@ -820,6 +820,13 @@ static std::vector<void*> graph_buffers(rt_ctx* ctx) {
     return v;
 }
 
+// Counts of the scene that a captured kernel holds by value: with another scene in
+// the same buffers it would take one hierarchy's records for the other's, or
+// boxes for beams that a scene loaded for the 8-wide layout does not have.
+static std::vector<int> graph_scene(const rt_ctx* ctx) {
+    return {ctx->n_tris, ctx->n_nodes, ctx->n_wnodes, ctx->n_bvh, ctx->n_big, ctx->n_mat, wide_layout(ctx), ctx->pk_ok};
+}
+
 int rt_graph_begin(rt_ctx* ctx) {
     CHECK_CTX(ctx);
     if (ctx->capturing) return set_err(ctx, RT_ERR_INVALID_ARG, "graph_begin: already capturing");
@@ -859,6 +866,7 @@ int rt_graph_end(rt_ctx* ctx) {
     e = cudaGraphInstantiate(&ctx->graph_exec, g, 0);
     cudaGraphDestroy(g);
     ctx->graph_bufs = graph_buffers(ctx);
+    ctx->graph_scene = graph_scene(ctx);
     if (e != cudaSuccess) {
         ctx->graph_exec = nullptr;
         return set_cuda(ctx, e, "cudaGraphInstantiate");
@@ -873,6 +881,10 @@ int rt_graph_launch(rt_ctx* ctx) {
         return set_err(ctx, RT_ERR_NOT_READY,
                        "graph_launch: a buffer the graph uses was reallocated since capture (larger scene, "
                        "devices or ray count); capture the graph again");
+    if (graph_scene(ctx) != ctx->graph_scene)
+        return set_err(ctx, RT_ERR_NOT_READY,
+                       "graph_launch: the scene's triangle, node or material counts or its layout changed since "
+                       "capture; capture the graph again");
     RT_TRY(cudaGraphLaunch(ctx->graph_exec, ctx->stream));
     ctx->launches += ctx->graph_kernels;
     return RT_OK;

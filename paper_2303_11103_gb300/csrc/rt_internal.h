@@ -140,6 +140,7 @@ struct rt_ctx {
     cudaGraphExec_t graph_exec = nullptr;
     int64_t launches_at_begin = 0, graph_kernels = 0;
     std::vector<void*> graph_bufs;   // addresses of the buffers a graph may use, at capture
+    std::vector<int> graph_scene;    // the scene's counts that its kernels hold
 };
 
 // Bracket one kernel launch: counts it and, when profiling, records CUDA
