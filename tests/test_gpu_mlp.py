@@ -188,7 +188,9 @@ def test_train_step_shapes(F, W, L, B, first):
                                      (32, 64, 2, 128 * 153),    # the same over a second tile
                                      (64, 64, 8, 256),
                                      (32, 128, 1, 128 * 153),   # one layer, a second tile
-                                     (32, 256, 1, 128)])
+                                     (32, 256, 1, 128),
+                                     (256, 64, 2, 256),         # eight chunks of features into one of columns
+                                     (4, 64, 2, 256)])          # the fewest features, layer by layer
 def test_train_step_chunks(F, W, L, B):
     """One fused step where warps share a chunk or two stored-only chunks follow each other."""
     test_train_step_shapes(F, W, L, B, 0)
